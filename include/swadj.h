@@ -137,7 +137,8 @@ int swa_get_time(swa_grid *grid, double *t, double *dt_next,
 
 /*
  * Launch shape of the FP32 2D step kernel: the height in rows of the strip a
- * warp walks, 16, 32 or 64 (0 restores the default, 32).  Results do not
+ * warp walks, 16, 32 or 64 (0 restores the default, chosen from the grid size
+ * so that the strips fill the resident warps).  Results do not
  * depend on it; throughput does (the autotuner picks it per grid size).
  * FP64 and 1D grids ignore it.
  */

@@ -211,8 +211,7 @@ static int grid_max_blocks(const swa_grid_desc *d) {
     int c;
     if (d->precision == SWA_FP32) {
         FwdParams<float> p{};
-        p.nx = d->nx; p.ny = d->ny; p.two_d = 1; p.fwd_rows = SWA_MIN_STRIP_ROWS;
-        if (fwd_step_blocks<float>(p) > b) b = fwd_step_blocks<float>(p);
+        p.nx = d->nx; p.ny = d->ny; p.two_d = 1;
         c = fwd_ctu_blocks<float>(p);
     } else {
         FwdParams<double> p{};

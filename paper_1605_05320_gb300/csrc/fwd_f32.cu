@@ -19,7 +19,8 @@ namespace f32 {
 
 
 // 2D grids: persistent warps take work units from the clock's counter, one
-// unit a strip of 28 output columns by `rows` rows, in row-major order.
+// unit a strip of 28 output columns by `rows` rows, in row-major order, then
+// the gauges of a recorded step, 32 a unit.
 // Where the ocean is at rest a unit costs little (strips.cuh), so units are
 // short and taken as warps free up: the active part of the domain spreads
 // over every SM instead of over the few warps whose strips it crosses.
@@ -37,11 +38,10 @@ __global__ void __launch_bounds__(strip::kThreads, 4)
                            t_now, dt))
         return;
     const int cur = s_cur;
-    // with gauge recording, the last block first samples the state the step
-    // starts from (the others write the other buffer)
-    if (p.gauges.n > 0 && blockIdx.x == gridDim.x - 1)
-        record_gauges<float, strip::kThreads>(p.gauges, p.q[cur][0], p.bath, p.nx, p.ny, 1,
-                                              t_now);
+    // with gauge recording, the warps that first run out of strips sample the
+    // state the step starts from, 32 gauges each (the strips write the other
+    // buffer)
+    const int ngroups = p.gauges.n > 0 ? (p.gauges.n + 31) / 32 : 0;
     const int nsx = (p.nx + strip::kOut - 1) / strip::kOut;
     strip::View v;
     v.q0 = p.q[cur][0]; v.q1 = p.q[cur][1]; v.q2 = p.q[cur][2]; v.hb = p.bath;
@@ -57,7 +57,12 @@ __global__ void __launch_bounds__(strip::kThreads, 4)
         int u = 0;
         if (lane == 0) u = (int)atomicAdd(&p.clk->work, 1u);
         u = __shfl_sync(0xffffffffu, u, 0);
-        if (u >= nunits) break;
+        if (u >= nunits) {
+            if (u >= nunits + ngroups) break;
+            record_gauge_group<float>(p.gauges, p.q[cur][0], p.bath, p.nx, p.ny, 1, p.clk,
+                                      u - nunits);
+            continue;
+        }
         const int sy = u / nsx, sx = u - sy * nsx;
         // A unit that had waves at an earlier step keeps them (the ocean does
         // not return exactly to rest behind a wave): it skips the quiet scan.
@@ -76,6 +81,7 @@ __global__ void __launch_bounds__(strip::kThreads, 4)
     if (bad) atomicOr(p.err, ERR_UNSTABLE);
     fwave::finish_step<strip::kThreads>(p.clk, p.partial, p.nblocks, p.cfl, smax, red, &am_last,
                                         t_now, dt, cur);
+    if (ngroups > 0 && threadIdx.x == 0 && am_last) *p.gauges.row += 1;
 }
 
 // 1D grids: one thread per cell, solving the four edges it needs itself
@@ -153,9 +159,12 @@ __global__ void rest_cfl_table(FwdParams<float> p, float *tab) {
 
 }  // namespace f32
 
-// Entries of the unit map: units of the lowest strip height (16 rows).
+// Lowest height of a work unit in rows.
+constexpr int kMinUnitRows = 4;
+
+// Entries of the unit map: units of the lowest height.
 int fwd_f32_unit_map_bytes(int nx, int ny) {
-    return ((nx + strip::kOut - 1) / strip::kOut) * ((ny + 15) / 16);
+    return ((nx + strip::kOut - 1) / strip::kOut) * ((ny + kMinUnitRows - 1) / kMinUnitRows);
 }
 
 size_t fwd_f32_rest_table_floats(int nx, int ny) {
@@ -170,19 +179,9 @@ int fwd_f32_rest_table(const FwdParams<float> &p, float *tab, cudaStream_t st) {
     return swadj_host::cuda_check(cudaGetLastError(), "rest_cfl_table");
 }
 
-// Rows of a work unit of the FP32 2D step: the requested strip height (16,
-// 32 or 64), else kUnitRows.  All heights give the same results.
-constexpr int kUnitRows = 32;
 // Persistent blocks at most (reduction slots of the grid workspace).
 constexpr int kMaxStepBlocks = 4096;
 
-static int unit_rows(const FwdParams<float> &p) {
-    return (p.fwd_rows == 16 || p.fwd_rows == 32 || p.fwd_rows == 64) ? p.fwd_rows : kUnitRows;
-}
-
-static int strip_units(int nx, int ny, int rows) {
-    return ((nx + strip::kOut - 1) / strip::kOut) * ((ny + rows - 1) / rows);
-}
 
 // Blocks of one resident wave of the strip kernel on the current device.
 static int resident_blocks() {
@@ -199,6 +198,36 @@ static int resident_blocks() {
     return blocks;
 }
 
+static int strip_units(int nx, int ny, int rows) {
+    return ((nx + strip::kOut - 1) / strip::kOut) * ((ny + rows - 1) / rows);
+}
+
+// Rows of a work unit of the FP32 2D step: the requested strip height (16,
+// 32 or 64), else the lowest height (at least kMinUnitRows) whose units are
+// no more than k times the resident warps, for the smallest k that needs no
+// more than kMaxUnitRows rows.  A unit walks its rows one after the other,
+// 0.58 us each when its warp is alone on its scheduler, so a grid of fewer
+// units than warps is latency-bound and takes the lowest units that still
+// fill the warps; a grid of many units wants them high (each walks four
+// halo rows more) and a whole number of rounds.  All heights give the same
+// results.
+// Measured, us per step, 32 rows / this rule (rest outside the source, waves
+// everywhere): 64^2 28.7 / 12.3 both; 512^2 26.9 / 15.7 and 28.1 / 18.1; 1024^2
+// 30.1 / 23.9 and 32.8 / 28.7; 1500^2 (34 rows) 33.9 / 35.4 and 53.3 / 44.4;
+// 2048^2 keeps 32; 4096^2 (36 rows) 84.3 / 86.1 and 258 / 248.
+constexpr int kMaxUnitRows = 36;
+static int unit_rows(const FwdParams<float> &p) {
+    if (p.fwd_rows > 0) return p.fwd_rows;
+    const long long warps = (long long)resident_blocks() * (strip::kThreads / 32);
+    const int nsx = (p.nx + strip::kOut - 1) / strip::kOut;
+    long long k = ((long long)nsx + warps - 1) / warps;
+    for (;; k++) {
+        const long long bands = k * warps / nsx;
+        const long long rows = (p.ny + bands - 1) / bands;
+        if (rows <= kMaxUnitRows) return rows > kMinUnitRows ? (int)rows : kMinUnitRows;
+    }
+}
+
 template <>
 int fwd_launch_step<float>(const FwdParams<float> &p0, cudaStream_t st) {
     FwdParams<float> p = p0;
@@ -209,7 +238,7 @@ int fwd_launch_step<float>(const FwdParams<float> &p0, cudaStream_t st) {
         int blocks = (units + wpb - 1) / wpb;
         const int wave = resident_blocks();
         if (blocks > wave) blocks = wave;
-        p.nblocks = blocks + (p.gauges.n > 0 ? 1 : 0);
+        p.nblocks = blocks;
         if (p.order == 2)
             f32::fwd_f32_strips<2><<<p.nblocks, strip::kThreads, 0, st>>>(p, rows, units);
         else
@@ -225,10 +254,10 @@ int fwd_launch_step<float>(const FwdParams<float> &p0, cudaStream_t st) {
 template <>
 int fwd_step_blocks<float>(const FwdParams<float> &p) {
     // one reduction slot per block: at most one block per 4 units (of the
-    // lowest height), at most kMaxStepBlocks, and the gauge block
+    // lowest height), at most kMaxStepBlocks
     if (p.two_d) {
-        const int b = (strip_units(p.nx, p.ny, 16) + 3) / 4;
-        return (b < kMaxStepBlocks ? b : kMaxStepBlocks) + 1;
+        const int b = (strip_units(p.nx, p.ny, kMinUnitRows) + 3) / 4;
+        return b < kMaxStepBlocks ? b : kMaxStepBlocks;
     }
     return (p.nx + 255) / 256;
 }

@@ -87,4 +87,20 @@ __device__ __forceinline__ void record_gauges(const GaugeRec &g, const R *q0, co
     if (tid == 0 && g.times) g.times[r] = t;
 }
 
+// The same for one warp: gauges 32 group .. 32 group + 31 of the row at
+// *g.row, the time from the device clock (group 0).  The caller advances the
+// row counter once every group of the step is written.
+template <typename R>
+__device__ __forceinline__ void record_gauge_group(const GaugeRec &g, const R *q0, const R *bath,
+                                                   int nx, int ny, int two_d,
+                                                   const DevClock *clk, int group) {
+    const long long r = *(volatile const long long *)g.row;
+    if (r >= g.cap) return;
+    const int lane = threadIdx.x & 31, k = group * 32 + lane;
+    if (k < g.n)
+        g.series[r * g.n + k] = gauge_eta<R>(q0, bath, nx, ny, two_d, g.x_lo, g.y_lo, g.dx,
+                                             g.dy, g.xy[2 * k], g.xy[2 * k + 1]);
+    if (group == 0 && lane == 0 && g.times) g.times[r] = ((volatile const DevClock *)clk)->t;
+}
+
 }  // namespace swadj
