@@ -75,8 +75,8 @@ __global__ void __launch_bounds__(strip::kThreads, 4)
         }
         // Units with waves take the full path: quiet units cover the ocean
         // at rest, and the strip loop without its row skipping is leaner.
-        strip::strip_unit(v, sx * strip::kOut, sy * rows, rows, s_nu[0], s_nu[1], p.g, ORD,
-                          ring[threadIdx.x >> 5], smax, bad, false);
+        strip::strip_unit<ORD, 2>(v, sx * strip::kOut, sy * rows, rows, s_nu[0], s_nu[1], p.g,
+                               ring[threadIdx.x >> 5], smax, bad);
     }
     if (bad) atomicOr(p.err, ERR_UNSTABLE);
     fwave::finish_step<strip::kThreads>(p.clk, p.partial, p.nblocks, p.cfl, smax, red, &am_last,
@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(256) fwd_f32_1d(FwdParams<float> p) {
     float sm = 0.f;
     bool bad = false;
     if (i < p.nx) {
-        fp::Cell<float> c[5];
+        fp::Cell c[5];
 #pragma unroll
         for (int k = 0; k < 5; k++) {
             bool fx;
@@ -113,12 +113,12 @@ __global__ void __launch_bounds__(256) fwd_f32_1d(FwdParams<float> p) {
             c[k] = fp::derive(eta, fp::add(eta, p.bath[ci]), mu, 0.f);
         }
         const float gh = 0.5f * g;
-        fp::Edge<float> w[4];
+        fp::Edge w[4];
 #pragma unroll
         for (int k = 0; k < 4; k++) w[k] = fp::solve(gh, c[k], c[k + 1]);
-        const fp::Net<float> n0 =
+        const fp::Net n0 =
             fp::net3(w[0], w[1], w[2], nux, p.order, fp::subsonic(w[1].s1, w[1].s3));
-        const fp::Net<float> n1 =
+        const fp::Net n1 =
             fp::net3(w[1], w[2], w[3], nux, p.order, fp::subsonic(w[2].s1, w[2].s3));
         const float d0 = fp::mul(-nux, fp::add(n0.R0, n1.L0));
         const float ne = fp::add(c[2].eta, d0);

@@ -140,7 +140,7 @@ __device__ __forceinline__ CellRaw raw_at(const strip::View &v, int i, int j,
 }
 
 // x-frame cell data of cell (i, j)
-__device__ __forceinline__ fp::Cell<float> xcell(const strip::View &v, int i, int j,
+__device__ __forceinline__ fp::Cell xcell(const strip::View &v, int i, int j,
                                                  const RingCtx *rc = nullptr) {
     const CellRaw c = raw_at(v, i, j, rc);
     return fp::derive(c.eta, fp::add(c.eta, c.hb), c.mu, c.mv);
@@ -148,21 +148,21 @@ __device__ __forceinline__ fp::Cell<float> xcell(const strip::View &v, int i, in
 
 // the x-swept cell (i, j) in the y frame, as the strip kernel's x-sweep
 // leaves it
-__device__ __forceinline__ fp::Cell<float> xswept(const strip::View &v, int i, int j, float gh,
+__device__ __forceinline__ fp::Cell xswept(const strip::View &v, int i, int j, float gh,
                                                   float nux, int order,
                                                   const RingCtx *rc = nullptr) {
-    fp::Cell<float> c[5];
+    fp::Cell c[5];
 #pragma unroll
     for (int k = 0; k < 5; k++) c[k] = xcell(v, i - 2 + k, j, rc);
-    fp::Edge<float> w[4];
+    fp::Edge w[4];
 #pragma unroll
     for (int k = 0; k < 4; k++) w[k] = fp::solve(gh, c[k], c[k + 1]);
-    const fp::Net<float> nl = fp::net3(w[0], w[1], w[2], nux, order, fp::subsonic(w[1].s1, w[1].s3));
-    const fp::Net<float> nr = fp::net3(w[1], w[2], w[3], nux, order, fp::subsonic(w[2].s1, w[2].s3));
+    const fp::Net nl = fp::net3(w[0], w[1], w[2], nux, order, fp::subsonic(w[1].s1, w[1].s3));
+    const fp::Net nr = fp::net3(w[1], w[2], w[3], nux, order, fp::subsonic(w[2].s1, w[2].s3));
     const float d0 = fp::mul(-nux, fp::add(nl.R0, nr.L0));
     const float d1 = fp::mul(-nux, fp::add(nl.R1, nr.L1));
     const float d2 = fp::mul(-nux, fp::add(nl.R2, nr.L2));
-    const fp::Cell<float> &a = c[2];
+    const fp::Cell &a = c[2];
     return fp::derive(fp::add(a.eta, d0), fp::add(a.h, d0), fp::add(a.mt, d2), fp::add(a.mn, d1));
 }
 
@@ -177,18 +177,18 @@ __device__ __forceinline__ float group_flux(const strip::View &v, int i, int j, 
     using strip::dn;
     using strip::up;
     const int q = threadIdx.x & 3;
-    const fp::Cell<float> c =
+    const fp::Cell c =
         axis == 0 ? xcell(v, i + k0 + q, j, rc) : xswept(v, i, j + k0 + q, gh, nux, order, rc);
-    fp::Cell<float> n = c;
+    fp::Cell n = c;
     n.h = dn(c.h); n.mn = dn(c.mn); n.sq = dn(c.sq); n.su = dn(c.su); n.sv = dn(c.sv);
     n.P = dn(c.P); n.T = dn(c.T); n.eta = dn(c.eta);
-    const fp::Edge<float> w = fp::solve(gh, c, n);   // edge (q | q + 1)
-    fp::Edge<float> wl = w, wr = w;
+    const fp::Edge w = fp::solve(gh, c, n);   // edge (q | q + 1)
+    fp::Edge wl = w, wr = w;
     wl.s1 = up(w.s1); wl.s3 = up(w.s3); wl.vh = up(w.vh);
     wl.b1 = up(w.b1); wl.b2 = up(w.b2); wl.b3 = up(w.b3);
     wr.s1 = dn(w.s1); wr.s3 = dn(w.s3); wr.vh = dn(w.vh);
     wr.b1 = dn(w.b1); wr.b2 = dn(w.b2); wr.b3 = dn(w.b3);
-    const fp::Net<float> N =
+    const fp::Net N =
         fp::net3(wl, w, wr, axis == 0 ? nux : nuy, order, fp::subsonic(w.s1, w.s3));
     return fp::add(c.mn, N.L0);
 }
@@ -358,8 +358,8 @@ __global__ void __launch_bounds__(strip::kThreads, 4) level_strip_kernel(LevelPa
             if (strip::quiet_unit<false>(v, nullptr, 0, t.y, t.z, p.rows, p.g, smax)) continue;
             if ((threadIdx.x & 31) == 0) p.units[u].w = 1;
         }
-        strip::strip_unit(v, t.y, t.z, p.rows, s_nu[0], s_nu[1], p.g, ORD,
-                          ring[threadIdx.x >> 5], smax, bad);
+        strip::strip_unit<ORD, 1>(v, t.y, t.z, p.rows, s_nu[0], s_nu[1], p.g,
+                               ring[threadIdx.x >> 5], smax, bad);
     }
     if (p.rf.nfine + p.rf.ncoarse > 0) {
         // the warps with one strip fewer start on the refluxing tasks; the

@@ -44,10 +44,9 @@ __device__ __forceinline__ float up(float x) { return __shfl_up_sync(kFull, x, 1
 // the warp may take the SUB form, given this lane's edge (the nets of edges
 // (1|2) .. (29|30) are used).
 struct Nb1 {
-    typedef float V;
     static __device__ __forceinline__ float l(float x) { return up(x); }
     static __device__ __forceinline__ float r(float x) { return dn(x); }
-    static __device__ __forceinline__ bool ok(const fp::Edge<float> &w, int lane) {
+    static __device__ __forceinline__ bool ok(const fp::Edge &w, int lane) {
         return lane < 1 || lane > kLanes - 3 || fp::subsonic(w.s1, w.s3);
     }
 };
@@ -56,52 +55,54 @@ struct Nb1 {
 // limiter needs from the lanes beside it: in the SUB form only the upwind
 // values (wave 1 from the right edge, wave 3 from the left, both shear
 // strengths), otherwise both neighbours in full.
-template <class NB>
-__device__ __forceinline__ fp::Net<typename NB::V> xnet(const fp::Edge<typename NB::V> &w,
-                                                        typename NB::V nu, int order,
-                                                        bool all_sub) {
-    typedef typename NB::V V;
-    fp::Up<V> u1, u3;
-    if (all_sub) {
-        V b2l = w.b2, b2r = w.b2;
-        if (order >= 2) {
+template <class NB, bool SUB, int ORD>
+__device__ __forceinline__ fp::Net xnet(const fp::Edge &w,
+                                                        float nu) {
+    fp::Up u1 = {}, u3 = {};
+    if (SUB) {
+        float b2l = w.b2, b2r = w.b2;
+        if (ORD >= 2) {
             u1.s = NB::r(w.s1); u1.vh = NB::r(w.vh); u1.b = NB::r(w.b1);
             u3.s = NB::l(w.s3); u3.vh = NB::l(w.vh); u3.b = NB::l(w.b3);
             b2l = NB::l(w.b2); b2r = NB::r(w.b2);
         }
-        return fp::net<V, true>(w, u1, u3, b2l, b2r, nu, order);
+        return fp::net<true>(w, u1, u3, b2l, b2r, nu, ORD);
     }
-    fp::Edge<V> wl = w, wr = w;
-    if (order >= 2) {
+    fp::Edge wl = w, wr = w;
+    if (ORD >= 2) {
         wl.s1 = NB::l(w.s1); wl.s3 = NB::l(w.s3); wl.vh = NB::l(w.vh);
         wl.b1 = NB::l(w.b1); wl.b2 = NB::l(w.b2); wl.b3 = NB::l(w.b3);
         wr.s1 = NB::r(w.s1); wr.s3 = NB::r(w.s3); wr.vh = NB::r(w.vh);
         wr.b1 = NB::r(w.b1); wr.b2 = NB::r(w.b2); wr.b3 = NB::r(w.b3);
     }
     fp::upwind(w, wl, wr, u1, u3);
-    return fp::net<V, false>(w, u1, u3, wl.b2, wr.b2, nu, order);
+    return fp::net<false>(w, u1, u3, wl.b2, wr.b2, nu, ORD);
 }
 
-// x-sweep of one row held across the warp (x frame: mn = hu, mt = hv).
-// Returns the x-swept cell(s) in the y frame (mn = hv).  Lanes see their
-// right neighbour cells through NB::r; a cell takes R of the edge on its left
-// and L of the edge on its right.
+// The x-edge(s) a lane solves, between its cell and its right neighbour
+// (x frame: mn = hu, mt = hv).
 template <class NB>
-__device__ __forceinline__ fp::Cell<typename NB::V> xsweep(const fp::Cell<typename NB::V> &c,
-                                                           typename NB::V g_half, float nux,
-                                                           int order, int lane) {
-    typedef typename NB::V V;
-    fp::Cell<V> r;
+__device__ __forceinline__ fp::Edge xsolve(const fp::Cell &c,
+                                                           float g_half) {
+    fp::Cell r;
     r.h = NB::r(c.h); r.mn = NB::r(c.mn); r.mt = c.mt; r.sq = NB::r(c.sq);
     r.su = NB::r(c.su); r.sv = NB::r(c.sv); r.P = NB::r(c.P); r.T = NB::r(c.T);
     r.eta = NB::r(c.eta);
-    const fp::Edge<V> w = fp::solve(g_half, c, r);
-    const fp::Net<V> n =
-        xnet<NB>(w, fp::splat<V>(nux), order, __all_sync(kFull, NB::ok(w, lane)));
-    const V mnu = fp::splat<V>(-nux);
-    const V d0 = fp::mul(mnu, fp::add(NB::l(n.R0), n.L0));
-    const V d1 = fp::mul(mnu, fp::add(NB::l(n.R1), n.L1));
-    const V d2 = fp::mul(mnu, fp::add(NB::l(n.R2), n.L2));
+    return fp::solve(g_half, c, r);
+}
+
+// The x-swept cell(s) in the y frame (mn = hv) from a lane's cell c and its
+// edge w: a cell takes R of the edge on its left and L of the edge on its
+// right.
+template <class NB, bool SUB, int ORD>
+__device__ __forceinline__ fp::Cell xsweep(const fp::Cell &c,
+                                                           const fp::Edge &w,
+                                                           float nux) {
+    const fp::Net n = xnet<NB, SUB, ORD>(w, nux);
+    const float mnu = -nux;
+    const float d0 = fp::mul(mnu, fp::add(NB::l(n.R0), n.L0));
+    const float d1 = fp::mul(mnu, fp::add(NB::l(n.R1), n.L1));
+    const float d2 = fp::mul(mnu, fp::add(NB::l(n.R2), n.L2));
     return fp::derive(fp::add(c.eta, d0), fp::add(c.h, d0), fp::add(c.mt, d2),
                       fp::add(c.mn, d1));
 }
@@ -133,91 +134,67 @@ __device__ __forceinline__ void fetch_row(Ring &R, int slot, const View &v, int 
 // One strip of view v: output columns x0 .. x0 + 27 and rows y0 .. y0 +
 // rows - 1 (clipped to the view).  Called by all 32 lanes of a warp, with
 // the warp's own ring R.  Accumulates the CFL maximum of the new cells into
-// smax and sets bad on a non-positive depth or non-finite momentum.  skip:
-// take the exact shortcut of wave-free rows (false computes them in full,
-// with the same result).
+// smax and sets bad on a non-positive depth or non-finite momentum.
+//
+// The x-sweep of a row and the y-sweep of the row before it are independent
+// chains of shuffles, special-function operations and arithmetic; the loop
+// runs them side by side (row j is x-swept while the y-edge (j-2|j-1) is
+// solved and row j - 3 finished), in one block of code per form, so that a
+// warp has two chains in flight.
+// UNR: rows per pass of the loop.  Unrolling saves register moves but the
+// code of three rows and both forms no longer stays in the instruction
+// caches: at 4096^2 half covered by waves 1 / 2 / 3 rows take 199 / 201 / 215
+// us and everywhere 235 / 233 / 231; at 2048^2 everywhere 76.6 / 71.8 / 74.2;
+// the patch kernel, which spills registers at 2, takes 64 / 66 / 68.
+template <int ORD, int UNR>
 __device__ __forceinline__ void strip_unit(const View &v, int x0, int y0, int rows, float nux,
-                                           float nuy, float g, int order, Ring &R, float &smax,
-                                           bool &bad, bool skip = true) {
+                                           float nuy, float g, Ring &R, float &smax, bool &bad) {
+    typedef fp::Cell Cell;
+    typedef fp::Edge Edge;
     const int lane = threadIdx.x & 31;
     const int ylast = (y0 + rows < v.ny ? y0 + rows : v.ny) - 1;
     const int gi = x0 - 2 + lane;
-    bool fx, fy;
+    bool fx;
     const int col = ghost_index(gi, v.nx, v.bc.lo_x, v.bc.hi_x, &fx);
     const bool out = lane >= 2 && lane < kLanes - 2 && gi < v.nx;
     const float gh = 0.5f * g;
-    fp::Cell<float> A = {}, B = {};   // x-swept rows j-2, j-1 (y frame)
-    fp::Edge<float> W1 = {}, W2 = {};  // y-edges (j-3|j-2), (j-2|j-1)
-    fp::Net<float> N1 = {};            // net of edge (j-3|j-2)
-    // rest: bit k set when row j-k is exactly at rest (eta = hu = hv = 0) in
-    // every lane of the warp.  There every wave is exactly zero, so the
-    // x-sweep of such a row is the identity, an edge between two such rows
-    // has no waves, and a net whose three edges lie in such rows is zero:
-    // that work is skipped and its exact result used (the ocean ahead of a
-    // tsunami is at rest).  The record of a wave-free edge has zero
-    // strengths, so any limiter ratio formed with it is zero as well.
-    unsigned rest = 0;
-    fp::Edge<float> still = {};
-    still.s1 = -1.f;
-    still.s3 = 1.f;
     // strips away from the lower and upper boundary need no row mapping
     const bool yin = y0 - 2 >= 0 && ylast + 2 < v.ny;
     const int jend = ylast + 2;
     int jn = y0 - 2, sn = 0;   // next row to fetch and its ring slot
-#pragma unroll
-    for (int k = 0; k < kRing - 1; k++) {
+    int jr = y0 - 2, sc = 0;   // next row to read and its ring slot
+    auto fetch = [&]() {
         if (jn <= jend) {
+            bool fy;
             const int row = yin ? jn : ghost_index(jn, v.ny, v.bc.lo_y, v.bc.hi_y, &fy);
             fetch_row(R, sn, v, col, row, lane);
         }
         cp_commit();
         jn++;
         sn = (sn + 1) & (kRing - 1);
-    }
-    int sc = 0;   // ring slot of row j
-#pragma unroll 3
-    for (int j = y0 - 2; j <= jend; j++) {
-        if (jn <= jend) {
-            const int row = yin ? jn : ghost_index(jn, v.ny, v.bc.lo_y, v.bc.hi_y, &fy);
-            fetch_row(R, sn, v, col, row, lane);
-        }
-        cp_commit();
-        jn++;
-        sn = (sn + 1) & (kRing - 1);
-        cp_wait<kRing - 1>();   // row j has landed
-        fy = false;
-        if (!yin) ghost_index(j, v.ny, v.bc.lo_y, v.bc.hi_y, &fy);
-        Raw4 Rc;
-        Rc.eta = R.v[sc][0][lane];
-        const float mu = R.v[sc][1][lane], mv = R.v[sc][2][lane];
-        Rc.hb = R.v[sc][3][lane];
-        Rc.mu = fx ? -mu : mu;
-        Rc.mv = fy ? -mv : mv;
+    };
+    // the next row, in the x frame
+    auto load = [&]() -> Cell {
+        fetch();
+        cp_wait<kRing - 1>();   // row jr has landed
+        bool fy = false;
+        if (!yin) ghost_index(jr, v.ny, v.bc.lo_y, v.bc.hi_y, &fy);
+        const float eta = R.v[sc][0][lane], mu = R.v[sc][1][lane], mv = R.v[sc][2][lane];
+        const float hb = R.v[sc][3][lane];
+        jr++;
         sc = (sc + 1) & (kRing - 1);
-        const bool at_rest =
-            __all_sync(kFull, skip && Rc.eta == 0.f && Rc.mu == 0.f && Rc.mv == 0.f);
-        rest = (rest << 1) | (at_rest ? 1u : 0u);
-        const float h = fp::add(Rc.eta, Rc.hb);
-        const fp::Cell<float> C = at_rest
-                                      ? fp::derive(Rc.eta, h, Rc.mv, Rc.mu)
-                                      : xsweep<Nb1>(fp::derive(Rc.eta, h, Rc.mu, Rc.mv), gh, nux,
-                                                    order, lane);
-        fp::Edge<float> Wn = W2;
-        if (j >= y0 - 1) Wn = (rest & 3u) == 3u ? still : fp::solve(gh, B, C);   // edge (j-1|j)
-        fp::Net<float> N = {};
-        if (j >= y0 + 1 && (rest & 15u) != 15u) {   // net of edge (j-2|j-1)
-            const bool all_sub = __all_sync(kFull, !out || fp::subsonic(W2.s1, W2.s3));
-            N = fp::net3(W1, W2, Wn, nuy, order, all_sub);
-        }
-        if (j >= y0 + 2 && out) {
-            // y-sweep of row j-2: lower edge -> R of the previous net, upper
-            // edge -> L of this one (y frame: component 1 is hv, 2 is hu)
-            const float d0 = fp::mul(-nuy, fp::add(N1.R0, N.L0));
-            const float d1 = fp::mul(-nuy, fp::add(N1.R1, N.L1));
-            const float d2 = fp::mul(-nuy, fp::add(N1.R2, N.L2));
-            const float ne = fp::add(A.eta, d0), nmv = fp::add(A.mn, d1);
-            const float nmu = fp::add(A.mt, d2);
-            const size_t o = (size_t)(j - 2) * v.nx + gi;
+        return fp::derive(eta, fp::add(eta, hb), fx ? -mu : mu, fy ? -mv : mv);
+    };
+    // y-sweep of a row (A, y frame: component 1 is hv, 2 is hu): its lower
+    // edge -> R of the previous net, its upper edge -> L of this one
+    auto finish = [&](const Cell &A, const fp::Net &N1, const fp::Net &N, int j) {
+        const float d0 = fp::mul(-nuy, fp::add(N1.R0, N.L0));
+        const float d1 = fp::mul(-nuy, fp::add(N1.R1, N.L1));
+        const float d2 = fp::mul(-nuy, fp::add(N1.R2, N.L2));
+        const float ne = fp::add(A.eta, d0), nmv = fp::add(A.mn, d1);
+        const float nmu = fp::add(A.mt, d2);
+        if (out) {
+            const size_t o = (size_t)j * v.nx + gi;
             v.o0[o] = ne;
             v.o1[o] = nmu;
             v.o2[o] = nmv;
@@ -225,10 +202,43 @@ __device__ __forceinline__ void strip_unit(const View &v, int x0, int y0, int ro
             bad |= !(h > 0.f) || !isfinite(nmu) || !isfinite(nmv);
             smax = fmaxf(smax, cfl_f32(h, nmu, nmv, g, v.rdx, v.rdy, 1));
         }
-        A = B; B = C;
+    };
+#pragma unroll
+    for (int k = 0; k < kRing - 1; k++) fetch();
+    Cell A = {}, B = {}, C = {};   // x-swept rows j-3, j-2, j-1 (y frame)
+    Edge W1 = {}, W2 = {};         // y-edges (j-4|j-3), (j-3|j-2)
+#pragma unroll 1
+    for (int k = 0; k < 4; k++) {   // rows y0 - 2 .. y0 + 1
+        const Cell c = load();
+        const Edge w = xsolve<Nb1>(c, gh);
+        const Cell D = __all_sync(kFull, Nb1::ok(w, lane)) ? xsweep<Nb1, true, ORD>(c, w, nux)
+                                                           : xsweep<Nb1, false, ORD>(c, w, nux);
+        if (k == 1) W1 = fp::solve(gh, C, D);
+        if (k == 2) W2 = fp::solve(gh, C, D);
+        A = B; B = C; C = D;
+    }
+    fp::Net N1 = {};   // net of edge (j-4|j-3)
+#pragma unroll UNR
+    for (int j = y0 + 2; j <= jend; j++) {
+        const Cell c = load();
+        const Edge w = xsolve<Nb1>(c, gh);
+        const Edge Wn = fp::solve(gh, B, C);   // y-edge (j-2|j-1)
+        Cell D;
+        fp::Net N;
+        if (__all_sync(kFull, Nb1::ok(w, lane) && (!out || fp::subsonic(W2.s1, W2.s3)))) {
+            D = xsweep<Nb1, true, ORD>(c, w, nux);
+            N = fp::net3(W1, W2, Wn, nuy, ORD, true);
+            if (j > y0 + 2) finish(A, N1, N, j - 3);
+        } else {
+            D = xsweep<Nb1, false, ORD>(c, w, nux);
+            N = fp::net3(W1, W2, Wn, nuy, ORD, false);
+            if (j > y0 + 2) finish(A, N1, N, j - 3);
+        }
+        A = B; B = C; C = D;
         W1 = W2; W2 = Wn;
         N1 = N;
     }
+    finish(A, N1, fp::net3(W1, W2, fp::solve(gh, B, C), nuy, ORD, false), ylast);
 }
 
 // ------------------------------------------------------------ quiet units
