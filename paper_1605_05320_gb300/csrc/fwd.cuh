@@ -26,6 +26,7 @@ struct FwdParams {
     unsigned char *umap;     // FP32 2D grid: 1 = unit had waves at an earlier step
     int umap_n;              // entries of umap
     GaugeRec gauges;   // fused gauge recording (n = 0: off)
+    int keep_input;    // FP64 2D: 1 leaves the old state in place and writes the other buffer
     int wetdry;        // 1: the shore solver at dry and transonic edges
     R dry_tol;         // a cell with h <= dry_tol is dry
 };

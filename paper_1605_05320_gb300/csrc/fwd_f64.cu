@@ -6,6 +6,7 @@
 // through g*hhat*(eta_R - eta_L); matching rounding is what keeps the FP64
 // path within 1e-12 of the reference after thousands of steps.
 #include "ctu_kernels.cuh"
+#include "fwd_sweeps64.cuh"
 
 namespace swadj {
 
@@ -17,9 +18,57 @@ static int launch_step(FwdParams<R> p, cudaStream_t st) {
     return swadj_host::cuda_check(cudaGetLastError(), "fwd_step_kernel<double>");
 }
 
+// Cells per segment of a pass over `lines` lines of n cells.  A warp's FP64
+// operations are about 147 per cell and 280 for the ends of its segment; the
+// FP64 units (one per scheduler, 4 per SM) finish within about half a unit of
+// one another, and part of a running grid is usually still.  Segments of 2 /
+// 6 / 14 / 32 cells on 512^2 take 271 / 214 / 262 / 536 us per step (the rule
+// takes 7 and 6: 213), on 2048^2 3164 / 2213 / 1994 / 2164 (14: 2006).
+static int f64_segment(int lines, int n, int sms) {
+    const double groups = (lines + 31) / 32, schedulers = 4.0 * sms;
+    int best = n;
+    double best_cost = 1e300;
+    for (int seg = 2; seg < 130; seg++) {
+        const double rounds = groups * ((n + seg - 1) / seg) / schedulers;
+        const double cost = (rounds > 1.0 ? 0.75 * rounds + 0.5 : 1.2) * (147.0 * seg + 280.0);
+        if (cost < best_cost) { best_cost = cost; best = seg; }
+        if (seg >= n) break;
+    }
+    return best;
+}
+
+template <bool YPASS, bool WD>
+static int launch_sweep(const FwdParams<double> &p, int sms, cudaStream_t st) {
+    const int lines = YPASS ? p.nx : p.ny, n = YPASS ? p.ny : p.nx;
+    int seg = f64_segment(lines, n, sms);
+    const int units = ((lines + 31) / 32) * ((n + seg - 1) / seg);
+    const int wpb = s64::kThreads / 32;
+    int blocks = (units + wpb - 1) / wpb;
+    if (blocks > 2 * sms) blocks = 2 * sms;
+    if (p.order == 2)
+        s64::fwd_f64_sweep<YPASS, WD, 2><<<blocks, s64::kThreads, 0, st>>>(p, seg, units);
+    else
+        s64::fwd_f64_sweep<YPASS, WD, 1><<<blocks, s64::kThreads, 0, st>>>(p, seg, units);
+    return swadj_host::cuda_check(cudaGetLastError(), "fwd_f64_sweep");
+}
+
+template <bool WD>
+static int launch_sweeps(const FwdParams<double> &p, cudaStream_t st) {
+    static int sms = 0;
+    if (sms == 0) {
+        int dev = 0, n = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        sms = n > 0 ? n : 1;
+    }
+    const int rc = launch_sweep<false, WD>(p, sms, st);
+    return rc ? rc : launch_sweep<true, WD>(p, sms, st);
+}
+
 template <>
 int fwd_launch_step<double>(const FwdParams<double> &p, cudaStream_t st) {
-    if (p.two_d) return launch_step<double, false, true, 32, 4>(p, st);
+    if (p.two_d && p.keep_input) return launch_step<double, false, true, 32, 4>(p, st);
+    if (p.two_d) return launch_sweeps<false>(p, st);
     return launch_step<double, false, false, 128, 1>(p, st);
 }
 
@@ -31,7 +80,7 @@ int fwd_step_blocks<double>(const FwdParams<double> &p) {
 
 template <>
 int fwd_launch_wd<double>(const FwdParams<double> &p, cudaStream_t st) {
-    if (p.two_d) return launch_step<double, false, true, 32, 4, true>(p, st);
+    if (p.two_d) return launch_sweeps<true>(p, st);
     return launch_step<double, false, false, 128, 1, true>(p, st);
 }
 

@@ -433,6 +433,7 @@ fwd_step_kernel(FwdParams<R> p) {
             clk->nsteps = clk->nsteps + 1;
             clk->ticket = 0u;
             clk->work = 0u;
+            clk->work2 = 0u;
         }
     }
 }
@@ -496,6 +497,7 @@ __global__ void __launch_bounds__(256) clock_init_kernel(FwdParams<R> p, double 
             clk->nsteps = 0;
             clk->ticket = 0u;
             clk->work = 0u;
+            clk->work2 = 0u;
         }
     }
 }

@@ -110,6 +110,7 @@ int run_static(const swa_grid_desc *d, const void *const q_in[3], void *const q_
     p.clk = (DevClock *)scratch;
     p.partial = (double *)((unsigned char *)scratch + kStaticClockBytes);
     p.nblocks = blocks;
+    p.keep_input = 1;
     p.err = err;
     int rc2 = fwd_launch_step<R>(p, st);
     if (rc2 != SWA_OK || !smax_out) return rc2;

@@ -19,6 +19,7 @@ struct DevClock {
     int cur;            // buffer index holding Q^n
     unsigned int ticket;  // last-block-done counter, 0 between launches
     unsigned int work;    // next work unit of a persistent step kernel, 0 between launches
+    unsigned int work2;   // the same for the second pass of a step in two passes
     double smax;        // s_max(Q^n)
 };
 
