@@ -32,6 +32,10 @@ struct AdjParams {
     int umap_n;
 };
 
+// One step (two with two_steps).  The new state is in dst, except that an
+// FP64 2D step of a size for which adj_f64_sweeps holds leaves it in src's
+// buffers (dst holds the y-swept state).
+bool adj_f64_sweeps(int nx, int ny);
 template <typename R>
 int adj_launch_step(const AdjParams<R> &p, cudaStream_t st);
 // entries of the FP32 2D adjoint's unit map

@@ -705,7 +705,8 @@ static int adj_steps(swa_adjoint *a, swa_snapstore *s, int ns, cudaStream_t st) 
         TRY(adj_launch_step<float>(p, st));
     }
     if (s) TRY(env_fold(s, s->count, st));
-    a->cur ^= 1;
+    if (!(a->d.precision == SWA_FP64 && a->d.ndim == 2 && adj_f64_sweeps(a->d.nx, a->d.ny)))
+        a->cur ^= 1;
     a->steps_done += ns;
     if (s) { s->tau_host.push_back(tau); s->count++; }
     return SWA_OK;

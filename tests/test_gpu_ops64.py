@@ -60,3 +60,31 @@ def test_sweeps_match_the_oracle_bit_for_bit(nx, ny, order, bc, wetdry):
     assert np.array_equal(st["h"], h)
     assert np.array_equal(st["hu"], u)
     assert np.array_equal(st["hv"], v)
+
+
+@pytest.mark.parametrize("nx,ny,order,bc", [(161, 130, 2, (0, 0, 0, 0)), (3, 700, 1, (1, 1, 1, 1)),
+                                            (700, 33, 2, (1, 0, 0, 1)), (2, 650, 2, (0, 1, 1, 0))])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_adjoint_sweeps_match_the_oracle_bit_for_bit(nx, ny, order, bc, precision):
+    """Sizes that take the adjoint's sweep passes, with an island, snapshots
+    in both storage types."""
+    B.build()
+    from paper_1605_05320_gb300 import swadj as S
+    S.load()
+    sc = synth.small_2d(nx, ny, seed=nx + ny, L=nx * 5e3)
+    Bt = sc.B.copy()
+    Bt[(np.arange(nx * ny) % 61) == 17] = 2.0
+    t_f = 40 * 0.75 * sc.grid.dx / np.sqrt(9.81 * 4000.0)
+    d = S.make_desc(2, nx, ny, 0.0, 0.0, sc.grid.dx, sc.grid.dy, precision=S.SWA_FP64,
+                    order=order, bc=bc)
+    adj = S.Adjoint(d, Bt, sc.phi, t_f)
+    store = S.SnapStore(adj, adj.info()[0] // 7 + 3, precision)
+    store.run_adjoint(7)
+    og = O.Grid.from_spec(sc.grid, order=order, bc=bc)
+    snaps, tau, N, _ = O.adj_run(og, np.maximum(-Bt, 0.0), sc.phi, t_f, 7)
+    assert adj.info()[0] == N
+    assert np.array_equal(adj.get_state().ravel(), snaps[-1].ravel())
+    assert np.array_equal(store.info()[1], np.asarray(tau))
+    esz, dt = (8, torch.float64) if precision == S.SWA_FP64 else (4, torch.float32)
+    got = store.ws[:snaps.size * esz].view(dt).cpu().numpy()
+    assert np.array_equal(got, snaps.ravel().astype(got.dtype))
