@@ -11,24 +11,28 @@
 // phi(theta) b is formed from (b, theta b) directly (zero for b = 0, where
 // the division form sets theta = 0).
 #include "adj_kernels.cuh"
+#include "packed.cuh"
 
 namespace swadj {
 namespace adjt {
 
+using fp::add;
+using fp::dup;
+using fp::f2;
+using fp::mk;
+using fp::mul;
+using fp::sub;
 __device__ __forceinline__ float rcpf(float x) { return rcp_ftz(x); }
-// Rounded single operations that the compiler never fuses (with explicit
-// fmaf the rounding of every expression is fixed in the source).
-__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
 
-// phi(theta) b for the MC limiter, r = theta b
-__device__ __forceinline__ float mc1(float b, float r) {
-    const float sg = b < 0.f ? -1.f : 1.f;
-    const float B = fabsf(b), Rr = mul(sg, r);
-    float m = fminf(mul(0.5f, add(B, Rr)), mul(2.f, B));
-    m = fminf(m, mul(2.f, Rr));
-    return mul(sg, fmaxf(m, 0.f));
+// phi(theta) b for the MC limiter, r = theta b, of a pair of waves: (b + r)/2
+// limited to [-m, m], m = 2 min(|b|, |r|) where b and r have one sign and 0
+// where they do not
+__device__ __forceinline__ float clamp_to(float t, float m) { return fmaxf(fminf(t, m), -m); }
+__device__ __forceinline__ f2 mc2(f2 b, f2 r) {
+    const f2 t = mul(dup(0.5f), add(b, r));
+    const f2 m = mul(dup(2.f), mk(fmaxf(fp::min_xorsign(b.x, r.x), 0.f),
+                                  fmaxf(fp::min_xorsign(b.y, r.y), 0.f)));
+    return mk(clamp_to(t.x, m.x), clamp_to(t.y, m.y));
 }
 
 struct EdgeA {   // waves of one edge: strengths and the (substituted) speeds
@@ -56,8 +60,9 @@ __device__ __forceinline__ EdgeA solve_a(float eL, float mL, float cL, float eR,
     const float d1 = fmaf(mul(cL, cL), mL, -mul(mul(cR, cR), mR));
     const float d2 = sub(eL, eR);
     const float rs = rcpf(add(cL, cR));
-    w.b1 = mul(fmaf(cR, d2, d1), rs);
-    w.b2 = mul(fmaf(cL, d2, -d1), rs);
+    const f2 b = mul(fma(mk(cR, cL), dup(d2), mk(d1, -d1)), dup(rs));
+    w.b1 = b.x;
+    w.b2 = b.y;
     w.cl = cL;
     w.cr = cR;
     return w;
@@ -69,24 +74,28 @@ __device__ __forceinline__ EdgeA solve_a(float eL, float mL, float cL, float eR,
 template <bool DRY = true>
 __device__ __forceinline__ float4 net_a(const EdgeA &wl, const EdgeA &w, const EdgeA &wr,
                                         float nu, int order) {
-    float F0 = 0.f, F1 = 0.f;
+    const f2 b = mk(w.b1, w.b2), c = mk(w.cl, w.cr);
+    float L0 = mul(w.b1, w.cl), R0 = -mul(w.b2, w.cr);
+    f2 q1 = b;   // (L1, R1)
     if (order >= 2 && (!DRY || !w.wall)) {
         // wave 1 (speed -cl) is upwinded from the right edge, wave 2 (+cr)
         // from the left edge
-        const float r1 = mul(mul(wr.b1, fmaf(wr.cl, w.cl, 1.f)), rcpf(fmaf(w.cl, w.cl, 1.f)));
-        const float r2 = mul(mul(wl.b2, fmaf(wl.cr, w.cr, 1.f)), rcpf(fmaf(w.cr, w.cr, 1.f)));
-        const float k1 = mul(mul(-0.5f, fmaf(-nu, w.cl, 1.f)), mc1(w.b1, r1));
-        const float k2 = mul(mul(0.5f, fmaf(-nu, w.cr, 1.f)), mc1(w.b2, r2));
-        F0 = fmaf(k1, w.cl, -mul(k2, w.cr));
-        F1 = add(k1, k2);
+        const f2 m = fma(c, c, dup(1.f));
+        const f2 r = mul(mul(mk(wr.b1, wl.b2), fma(mk(wr.cl, wl.cr), c, dup(1.f))),
+                         mk(rcpf(m.x), rcpf(m.y)));
+        const f2 k = mul(mul(mk(-0.5f, 0.5f), fma(dup(-nu), c, dup(1.f))), mc2(b, r));
+        const float F0 = fmaf(k.x, w.cl, -mul(k.y, w.cr));
+        const float F1 = add(k.x, k.y);
+        L0 = fmaf(w.b1, w.cl, F0);
+        R0 = sub(R0, F0);
+        q1 = fma(dup(F1), mk(1.f, -1.f), b);
     }
-    return make_float4(fmaf(w.b1, w.cl, F0), add(w.b1, F1), sub(-mul(w.b2, w.cr), F0),
-                       sub(w.b2, F1));
+    return make_float4(L0, q1.x, R0, q1.y);
 }
 
 // ---------------------------------------------------------------- strips
 // A warp owns a strip of 32 columns (lanes) of which the middle 28 are its
-// output, and SH output rows, which it walks downwards.  The y-sweep runs in
+// output, and `rows` output rows, which it walks downwards.  The y-sweep runs in
 // registers with a sliding window over rows (each y-edge solved and limited
 // once); every y-swept row is then x-swept across the warp with shuffles
 // (each x-edge solved and limited once by the lane on its left).  Lanes 0-1
@@ -96,7 +105,8 @@ __device__ __forceinline__ float4 net_a(const EdgeA &wl, const EdgeA &w, const E
 // further down keeps one row of register prefetch.
 constexpr int kLanes = 32;
 constexpr int kOut = kLanes - 4;   // output columns per strip
-constexpr int kRows = 32;          // output rows per strip
+constexpr int kMinRows = 4;        // lowest strip in output rows
+constexpr int kMaxRows = 18;       // highest
 constexpr unsigned kFull = 0xffffffffu;
 
 struct CellA {
@@ -174,16 +184,16 @@ struct RingA {
 // DRY: the grid has dry cells (wall checks on); ORD: the order of the
 // scheme (1 or 2), fixed at compile time.
 template <bool DRY, int ORD>
-__global__ void __launch_bounds__(256, 4) adj_f32_strips(AdjParams<float> p) {
+__global__ void __launch_bounds__(256, 4) adj_f32_strips(AdjParams<float> p, int rows) {
     __shared__ RingA ring[8];   // one per warp of the 256-thread block
     const int lane = threadIdx.x & 31;
-    const int nsx = (p.nx + kOut - 1) / kOut, nsy = (p.ny + kRows - 1) / kRows;
+    const int nsx = (p.nx + kOut - 1) / kOut, nsy = (p.ny + rows - 1) / rows;
     const int unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if ((p.snap_f || p.snap_d) && blockIdx.x == 0 && threadIdx.x == 0) *p.tau_dev = p.tau_val;
     if (unit >= nsx * nsy) return;   // warp-uniform
     const int sy = unit / nsx, sx = unit - sy * nsx;
-    const int x0 = sx * kOut, y0 = sy * kRows;
-    const int ylast = (y0 + kRows < p.ny ? y0 + kRows : p.ny) - 1;
+    const int x0 = sx * kOut, y0 = sy * rows;
+    const int ylast = (y0 + rows < p.ny ? y0 + rows : p.ny) - 1;
     const int gi = x0 - 2 + lane;
     bool fx;
     const int col = ghost_index(gi, p.nx, p.bc.lo_x, p.bc.hi_x, &fx);
@@ -495,7 +505,34 @@ __global__ void __launch_bounds__(256, 3) adj_f32_strips2(AdjParams<float> p) {
 }  // namespace adjt
 
 int adj_f32_unit_map_bytes(int nx, int ny) {
-    return ((nx + adjt::kOut - 1) / adjt::kOut) * ((ny + adjt::kRows - 1) / adjt::kRows);
+    return ((nx + adjt::kOut - 1) / adjt::kOut) * ((ny + adjt::kMinRows - 1) / adjt::kMinRows);
+}
+
+// Rows of a strip: the lowest (at least kMinRows) whose strips are no more
+// than k times the resident warps, for the smallest k that needs no more than
+// kMaxRows rows.  A grid of fewer strips than warps is latency-bound (a warp
+// walks its rows one after the other) and takes the lowest strips that still
+// fill the warps; on larger grids low strips follow the front of the still
+// zero adjoint more closely, at the price of four halo rows each.
+// Measured, us per step late in the solve, 32 rows / this rule: 64^2 18.5 /
+// 6.3, 512^2 18.5 / 8.2, 1024^2 18.5 / 14.4; 2048^2 (16 rows) 38.9 / 36.4 and
+// 25.9 / 24.9 early (8 rows: 38.5 and 24.1, 64: 43.4 and 33.5); 4096^2 (18)
+// 82.8 / 80.5.
+static int adj_rows(int nx, int ny) {
+    static long long warps = 0;
+    if (warps == 0) {
+        int dev = 0, sms = 0, per_sm = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, adjt::adj_f32_strips<false, 2>,
+                                                      256, 0);
+        warps = 8LL * (sms > 0 ? sms : 1) * (per_sm > 0 ? per_sm : 1);
+    }
+    const int nsx = (nx + adjt::kOut - 1) / adjt::kOut;
+    for (long long k = (nsx + warps - 1) / warps;; k++) {
+        const long long bands = k * warps / nsx, rows = (ny + bands - 1) / bands;
+        if (rows <= adjt::kMaxRows) return rows > adjt::kMinRows ? (int)rows : adjt::kMinRows;
+    }
 }
 
 template <>
@@ -508,17 +545,15 @@ int adj_launch_step<float>(const AdjParams<float> &p, cudaStream_t st) {
         return swadj_host::cuda_check(cudaGetLastError(), "adj_f32_strips2");
     }
     if (p.two_d) {
+        const int rows = adj_rows(p.nx, p.ny);
         const long long units = (long long)((p.nx + adjt::kOut - 1) / adjt::kOut) *
-                                ((p.ny + adjt::kRows - 1) / adjt::kRows);
+                                ((p.ny + rows - 1) / rows);
         const unsigned blocks = (unsigned)((units + 7) / 8);
-        if (p.all_wet && p.order == 2)
-            adjt::adj_f32_strips<false, 2><<<blocks, 256, 0, st>>>(p);
-        else if (p.all_wet)
-            adjt::adj_f32_strips<false, 1><<<blocks, 256, 0, st>>>(p);
-        else if (p.order == 2)
-            adjt::adj_f32_strips<true, 2><<<blocks, 256, 0, st>>>(p);
-        else
-            adjt::adj_f32_strips<true, 1><<<blocks, 256, 0, st>>>(p);
+        auto kernel = p.all_wet ? (p.order == 2 ? adjt::adj_f32_strips<false, 2>
+                                                : adjt::adj_f32_strips<false, 1>)
+                                : (p.order == 2 ? adjt::adj_f32_strips<true, 2>
+                                                : adjt::adj_f32_strips<true, 1>);
+        kernel<<<blocks, 256, 0, st>>>(p, rows);
         return swadj_host::cuda_check(cudaGetLastError(), "adj_f32_strips");
     }
     dim3 grid((p.nx + 127) / 128, 1);

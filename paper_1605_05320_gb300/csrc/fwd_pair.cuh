@@ -28,63 +28,22 @@
 // 4096^2 with waves everywhere: 256 us per step with scalar operations, 231
 // to 235 us so.
 #pragma once
-#include "swadj_internal.cuh"
+#include "packed.cuh"
 
 namespace swadj {
 namespace fp {
 
-__device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float fma(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ float fms(float a, float b, float c) { return fmaf(a, b, -c); }   // ab - c
 __device__ __forceinline__ float fnma(float a, float b, float c) { return fmaf(-a, b, c); }  // c - ab
 __device__ __forceinline__ float rcp(float x) { return rcp_ftz(x); }
 __device__ __forceinline__ float rsq(float x) { return rsqrt_ftz(x); }
 
-// Two floats operated on by packed instructions.
-struct f2 {
-    float x, y;
-};
-__device__ __forceinline__ f2 mk(float x, float y) { f2 r; r.x = x; r.y = y; return r; }
-__device__ __forceinline__ f2 dup(float x) { return mk(x, x); }
-__device__ __forceinline__ f2 fma(f2 a, f2 b, f2 c) {
-    f2 r;
-    asm("{\n\t.reg .b64 a, b, c, d;\n\t"
-        "mov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\t"
-        "fma.rn.f32x2 d, a, b, c;\n\tmov.b64 {%0, %1}, d;\n\t}"
-        : "=f"(r.x), "=f"(r.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-    return r;
-}
-__device__ __forceinline__ f2 mul(f2 a, f2 b) {
-    f2 r;
-    asm("{\n\t.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
-        "mul.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
-        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return r;
-}
-__device__ __forceinline__ f2 add(f2 a, f2 b) {
-    f2 r;
-    asm("{\n\t.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
-        "add.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
-        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return r;
-}
-__device__ __forceinline__ f2 rcp(f2 x) { return mk(rcp_ftz(x.x), rcp_ftz(x.y)); }
-
 // sign(s) in {-1, 0, 1}
 __device__ __forceinline__ float sgn(float s) { return s > 0.f ? 1.f : (s < 0.f ? -1.f : 0.f); }
 // s > 0 ? a : b
 __device__ __forceinline__ float pick(float s, float a, float b) { return s > 0.f ? a : b; }
 __device__ __forceinline__ bool subsonic(float s1, float s3) { return s1 < 0.f && s3 > 0.f; }
-
-// min(|a|, |b|) with the product's sign
-__device__ __forceinline__ float min_xorsign(float a, float b) {
-    float r;
-    asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
-}
 
 // Half the MC-limited wave strength: phi(theta) b / 2 for the MC limiter
 // phi = max(0, min((1 + theta)/2, 2, 2 theta)), given b and r = theta b: (b +
