@@ -186,6 +186,7 @@ struct RingA {
 template <bool DRY, int ORD>
 __global__ void __launch_bounds__(256, 4) adj_f32_strips(AdjParams<float> p, int rows) {
     __shared__ RingA ring[8];   // one per warp of the 256-thread block
+    chain_begin();
     const int lane = threadIdx.x & 31;
     const int nsx = (p.nx + kOut - 1) / kOut, nsy = (p.ny + rows - 1) / rows;
     const int unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -427,6 +428,7 @@ __device__ __forceinline__ CellA ghost_row(int r, int ny, int bc_lo, int bc_hi, 
 }
 
 __global__ void __launch_bounds__(256, 3) adj_f32_strips2(AdjParams<float> p) {
+    chain_begin();
     const int lane = threadIdx.x & 31;
     const int nsx = (p.nx + kOut2 - 1) / kOut2, nsy = (p.ny + kRows2 - 1) / kRows2;
     const int unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -541,8 +543,8 @@ int adj_launch_step<float>(const AdjParams<float> &p, cudaStream_t st) {
         const long long units = (long long)((p.nx + adjt::kOut2 - 1) / adjt::kOut2) *
                                 ((p.ny + adjt::kRows2 - 1) / adjt::kRows2);
         const unsigned blocks = (unsigned)((units + 7) / 8);
-        adjt::adj_f32_strips2<<<blocks, 256, 0, st>>>(p);
-        return swadj_host::cuda_check(cudaGetLastError(), "adj_f32_strips2");
+        return swadj_host::cuda_check(launch_chained(adjt::adj_f32_strips2, blocks, 256, 0, st, p),
+                                      "adj_f32_strips2");
     }
     if (p.two_d) {
         const int rows = adj_rows(p.nx, p.ny);
@@ -553,12 +555,13 @@ int adj_launch_step<float>(const AdjParams<float> &p, cudaStream_t st) {
                                                 : adjt::adj_f32_strips<false, 1>)
                                 : (p.order == 2 ? adjt::adj_f32_strips<true, 2>
                                                 : adjt::adj_f32_strips<true, 1>);
-        kernel<<<blocks, 256, 0, st>>>(p, rows);
-        return swadj_host::cuda_check(cudaGetLastError(), "adj_f32_strips");
+        return swadj_host::cuda_check(launch_chained(kernel, blocks, 256, 0, st, p, rows),
+                                      "adj_f32_strips");
     }
     dim3 grid((p.nx + 127) / 128, 1);
-    adj_step_kernel<float, false, 128, 1><<<grid, dim3(128, 1), 0, st>>>(p);
-    return swadj_host::cuda_check(cudaGetLastError(), "adj_step_kernel<float>");
+    return swadj_host::cuda_check(
+        launch_chained(adj_step_kernel<float, false, 128, 1>, grid, dim3(128, 1), 0, st, p),
+        "adj_step_kernel<float>");
 }
 
 }  // namespace swadj

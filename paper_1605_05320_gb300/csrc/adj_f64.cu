@@ -8,8 +8,9 @@ namespace swadj {
 template <typename R, bool TWO_D, int TX, int TY>
 static int launch_adj(const AdjParams<R> &p, cudaStream_t st) {
     dim3 grid((p.nx + TX - 1) / TX, TWO_D ? (p.ny + TY - 1) / TY : 1);
-    adj_step_kernel<R, TWO_D, TX, TY><<<grid, dim3(TX, TY), 0, st>>>(p);
-    return swadj_host::cuda_check(cudaGetLastError(), "adj_step_kernel<double>");
+    return swadj_host::cuda_check(
+        launch_chained(adj_step_kernel<R, TWO_D, TX, TY>, grid, dim3(TX, TY), 0, st, p),
+        "adj_step_kernel<double>");
 }
 
 static int sm_count() {

@@ -102,6 +102,7 @@ __global__ void __launch_bounds__(TX *TY) adj_step_kernel(AdjParams<R> p) {
 
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int tid = tx + ty * TX;
+    chain_begin();
     const int nx = p.nx, ny = p.ny;
     const int i0 = blockIdx.x * TX - HX, j0 = blockIdx.y * TY - HY;
 

@@ -183,6 +183,7 @@ fwd_ctu_kernel(FwdParams<R> p) {
 
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int tid = tx + ty * TX;
+    chain_begin();
     volatile DevClock *clk = p.clk;
     const double t = clk->t;
     double dt = clk->dt_cfl;
@@ -379,8 +380,8 @@ int ctu_launch(FwdParams<R> p, cudaStream_t st, const char *name) {
     if (rc) return rc;
     dim3 grid((p.nx + TX - 1) / TX, (p.ny + TY - 1) / TY);
     p.nblocks = (int)(grid.x * grid.y);
-    fwd_ctu_kernel<R, PERT, TX, TY><<<grid, dim3(TX, TY), smem, st>>>(p);
-    return swadj_host::cuda_check(cudaGetLastError(), name);
+    return swadj_host::cuda_check(
+        launch_chained(fwd_ctu_kernel<R, PERT, TX, TY>, grid, dim3(TX, TY), smem, st, p), name);
 }
 
 template <int TX, int TY>

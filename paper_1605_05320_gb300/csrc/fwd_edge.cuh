@@ -13,6 +13,7 @@ namespace fwave {
 __device__ __forceinline__ bool begin_step(DevClock *clkp, double t_end, double dx, double dy,
                                            float *s_nu, int *s_cur, int *s_run, double &t_now,
                                            double &dt) {
+    chain_begin();
     if (threadIdx.x == 0) {
         volatile DevClock *clk = clkp;
         t_now = clk->t;

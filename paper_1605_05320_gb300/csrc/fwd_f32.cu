@@ -239,16 +239,15 @@ int fwd_launch_step<float>(const FwdParams<float> &p0, cudaStream_t st) {
         const int wave = resident_blocks();
         if (blocks > wave) blocks = wave;
         p.nblocks = blocks;
-        if (p.order == 2)
-            f32::fwd_f32_strips<2><<<p.nblocks, strip::kThreads, 0, st>>>(p, rows, units);
-        else
-            f32::fwd_f32_strips<1><<<p.nblocks, strip::kThreads, 0, st>>>(p, rows, units);
-        return swadj_host::cuda_check(cudaGetLastError(), "fwd_f32_strips");
+        return swadj_host::cuda_check(
+            launch_chained(p.order == 2 ? f32::fwd_f32_strips<2> : f32::fwd_f32_strips<1>,
+                           p.nblocks, strip::kThreads, 0, st, p, rows, units),
+            "fwd_f32_strips");
     }
     dim3 grid((p.nx + 255) / 256, 1);
     p.nblocks = (int)grid.x;
-    f32::fwd_f32_1d<<<grid, 256, 0, st>>>(p);
-    return swadj_host::cuda_check(cudaGetLastError(), "fwd_f32_1d");
+    return swadj_host::cuda_check(launch_chained(f32::fwd_f32_1d, grid, 256, 0, st, p),
+                                  "fwd_f32_1d");
 }
 
 template <>
@@ -270,13 +269,18 @@ int fwd_launch_wd<float>(const FwdParams<float> &p0, cudaStream_t st) {
     if (p.two_d) {
         dim3 grid((p.nx + 31) / 32, (p.ny + 3) / 4);
         p.nblocks = (int)(grid.x * grid.y);
-        fwd_step_kernel<float, true, true, 32, 4, true><<<grid, dim3(32, 4), 0, st>>>(p);
+        return swadj_host::cuda_check(
+            launch_chained(fwd_step_kernel<float, true, true, 32, 4, true>, grid, dim3(32, 4), 0,
+                           st, p),
+            "fwd_step_kernel<float, wet/dry>");
     } else {
         dim3 grid((p.nx + 127) / 128, 1);
         p.nblocks = (int)grid.x;
-        fwd_step_kernel<float, true, false, 128, 1, true><<<grid, dim3(128, 1), 0, st>>>(p);
+        return swadj_host::cuda_check(
+            launch_chained(fwd_step_kernel<float, true, false, 128, 1, true>, grid, dim3(128, 1),
+                           0, st, p),
+            "fwd_step_kernel<float, wet/dry>");
     }
-    return swadj_host::cuda_check(cudaGetLastError(), "fwd_step_kernel<float, wet/dry>");
 }
 
 template <>

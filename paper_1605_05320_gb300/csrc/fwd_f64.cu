@@ -14,8 +14,9 @@ template <typename R, bool PERT, bool TWO_D, int TX, int TY, bool WD = false>
 static int launch_step(FwdParams<R> p, cudaStream_t st) {
     dim3 grid((p.nx + TX - 1) / TX, TWO_D ? (p.ny + TY - 1) / TY : 1);
     p.nblocks = (int)(grid.x * grid.y);
-    fwd_step_kernel<R, PERT, TWO_D, TX, TY, WD><<<grid, dim3(TX, TY), 0, st>>>(p);
-    return swadj_host::cuda_check(cudaGetLastError(), "fwd_step_kernel<double>");
+    return swadj_host::cuda_check(
+        launch_chained(fwd_step_kernel<R, PERT, TWO_D, TX, TY, WD>, grid, dim3(TX, TY), 0, st, p),
+        "fwd_step_kernel<double>");
 }
 
 // Cells per segment of a pass over `lines` lines of n cells.  A warp's FP64

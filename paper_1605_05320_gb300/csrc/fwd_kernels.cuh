@@ -194,6 +194,7 @@ fwd_step_kernel(FwdParams<R> p) {
 
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int tid = tx + ty * TX;
+    chain_begin();
     volatile DevClock *clk = p.clk;
     const double t = clk->t;
     double dt = clk->dt_cfl;

@@ -857,6 +857,7 @@ struct FillParams {
 __global__ void __launch_bounds__(128) amr_fill_kernel(FillParams p) {
     __shared__ float s_a;
     __shared__ int s_fcur, s_pcur;
+    chain_begin();
     if (threadIdx.x == 0) {
         volatile const DevClock *lc = p.lclk, *pc = p.rf.pclk;
         double a = (lc->t - p.rf.t_p) / p.rf.dt_p;
@@ -918,6 +919,7 @@ struct AvgParams {
 // different cells.  Also checks that both levels reached the step's end.
 template <int R>
 __global__ void amr_avg_kernel(AvgParams p) {
+    chain_begin();
     volatile const DevClock *lc = p.lclk, *pc = p.pclk;
     __shared__ int s_fcur, s_pcur;
     if (threadIdx.x == 0) {
@@ -982,6 +984,7 @@ struct CoarseReflux {
 };
 
 __global__ void reflux_coarse_kernel(CoarseReflux p) {
+    chain_begin();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const double tol = 1e-12 * (fabs(p.t_n) > 1.0 ? fabs(p.t_n) : 1.0);
         bool ok = fabs(((volatile const DevClock *)p.cclk)->t - p.t_n) <= tol;
@@ -1291,14 +1294,14 @@ int amr_average(swa_amr *A, const GridRefs &c, int l, double t_end, bool reflux,
     p.err = swadj_host::error_word();
     const size_t n = (size_t)3 * V.navg + (size_t)p.ncfu;
     const unsigned ab = patches::ew_blocks(n > 0 ? n : 1);
+    void (*kernel)(amr::AvgParams) = amr::amr_avg_kernel<0>;
     switch (V.r) {
-        case 1: amr::amr_avg_kernel<1><<<ab, 256, 0, st>>>(p); break;
-        case 2: amr::amr_avg_kernel<2><<<ab, 256, 0, st>>>(p); break;
-        case 4: amr::amr_avg_kernel<4><<<ab, 256, 0, st>>>(p); break;
-        case 8: amr::amr_avg_kernel<8><<<ab, 256, 0, st>>>(p); break;
-        default: amr::amr_avg_kernel<0><<<ab, 256, 0, st>>>(p); break;
+        case 1: kernel = amr::amr_avg_kernel<1>; break;
+        case 2: kernel = amr::amr_avg_kernel<2>; break;
+        case 4: kernel = amr::amr_avg_kernel<4>; break;
+        case 8: kernel = amr::amr_avg_kernel<8>; break;
     }
-    return cuda_check(cudaGetLastError(), "amr_avg_kernel");
+    return cuda_check(launch_chained(kernel, ab, 256, 0, st, p), "amr_avg_kernel");
 }
 
 // Level l of the hierarchy over the parent step [t_p, t_p + dt_p]
@@ -1340,8 +1343,8 @@ int amr_run(swa_amr *A, const GridRefs &c, int l, double t_p, double dt_p, int m
         const double t_km1 = k == 1 ? t_p : t_p + dt_p * (double)(k - 1) / (double)r;
         for (int j = 0; j < launches; j++) {
             if (!fused) {
-                amr::amr_fill_kernel<<<fb, 128, 0, st>>>(f);
-                TRY(cuda_check(cudaGetLastError(), "amr_fill_kernel"));
+                TRY(cuda_check(launch_chained(amr::amr_fill_kernel, fb, 128, 0, st, f),
+                               "amr_fill_kernel"));
             }
             TRY(level_launch(A->fine, V.lev, 1, t_k, rf, st, fused ? &lf : nullptr));
         }
@@ -1507,8 +1510,8 @@ int swa_amr_step(swa_amr *A, double t_n, double dt_c, int max_launches, void *st
     q.nlev = A->L;
     q.err = swadj_host::error_word();
     const unsigned eb = (unsigned)(q.ncf > 0 ? (q.ncf + 31) / 32 : 1);   // 8 edges per warp
-    amr::reflux_coarse_kernel<<<eb, 128, 0, st>>>(q);
-    TRY(cuda_check(cudaGetLastError(), "reflux_coarse_kernel"));
+    TRY(cuda_check(launch_chained(amr::reflux_coarse_kernel, eb, 128, 0, st, q),
+                   "reflux_coarse_kernel"));
     TRY(swa_step_forward(A->coarse, 1, t_end, stream));
     TRY(amr_run(A, c, 1, t_n, dt_c, max_launches, reflux, st));
     return amr_average(A, c, 1, t_end, reflux, st);

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "chain.cuh"
 #include "swadj.h"
 
 namespace swadj {
@@ -50,13 +51,13 @@ __device__ __forceinline__ int ghost_index(int g, int n, int bc_lo, int bc_hi,
     return g;
 }
 
-// Read-only global load as volatile inline PTX: it stays ahead of the
+// Global load as volatile inline PTX: it stays ahead of the
 // barriers that follow it in program order, so a register prefetch of the
 // next tile is issued before the current tile's work instead of being moved
 // next to its first use.
 __device__ __forceinline__ float ld_early(const float *p) {
     float v;
-    asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
     return v;
 }
 
