@@ -357,7 +357,7 @@ int swa_grid_gauge_rows(const swa_grid *grid, long long *rows, void *stream);
  * cells from its own boundary conditions and no exchange between patches).
  * FP32 perturbation form only.  One swa_step_level call enqueues one
  * kernel launch per step whose resident warps walk the strips (28 columns x
- * 16 or 32 rows) of every patch of that level; results do not depend on the
+ * up to 36 rows) of every patch of that level; results do not depend on the
  * strip height.  All patches of a level share one time step, reduced on the
  * device from their CFL maxima (dt_l = cfl / max over the level's cells),
  * so a loop of level steps can be captured in a CUDA graph.
@@ -403,10 +403,11 @@ int swa_patches_get_time(swa_patchset *ps, int level, double *t, double *dt_next
  * strip height) and cells of a level (host bookkeeping). */
 int swa_patches_level_info(const swa_patchset *ps, int level, int *npatches,
                            int *ntiles, long long *ncells);
-/* Strip height of the level's kernel in rows: 16 or 32 (0 = default: 16
- * when the level's 16-row strips are no more than the warps the launch keeps
- * resident, else 32).  Results do not depend on it; throughput does (the
- * autotuner picks it). */
+/* Greatest strip height of the level's kernel in rows: 16 or 32 (0 = default:
+ * chosen at creation so that the level's strips fill a whole number of rounds
+ * of the warps the launch keeps resident).  A patch is cut into bands of equal
+ * height.  Results do not depend on it; throughput does (the autotuner picks
+ * it). */
 int swa_patches_set_tile_rows(swa_patchset *ps, int level, int rows);
 
 /* ============================== AMR glue ===================================

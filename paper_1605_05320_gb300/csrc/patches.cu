@@ -10,6 +10,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 #include <vector>
 
@@ -231,7 +232,7 @@ struct LevelReflux {
 struct LevelParams {
     const PatchDevice *table;
     int4 *units;         // (patch, x0, y0, hint): hint 1 = the strip has had waves
-    int nunits, rows;
+    int nunits, rows;    // rows: the greatest height of a strip
     DevClock *clk;
     double *partial;
     int nblocks;
@@ -244,17 +245,24 @@ struct LevelParams {
     int fill_on;
 };
 
+// Rows of a strip: a patch of ny rows is cut into the fewest bands of at most
+// `rows` rows, of equal height but for the last.
+__host__ __device__ __forceinline__ int strip_rows(int ny, int rows) {
+    const int bands = (ny + rows - 1) / rows;
+    return (ny + bands - 1) / bands;
+}
+
 // Fill the ring cells of patch pid inside the stencil window of the strip at
 // (x0, y0) (columns x0 - 2 .. x0 + 29, rows y0 - 2 .. the strip's last row +
 // 2, clipped to the array) in the current buffer, the warp's lanes taking
 // the window's cells in turn.  Strips of a patch share ring cells; each
 // writes the same value, so the writes of two strips agree, and a strip
 // reads only cells it has written itself.
-__device__ __noinline__ void fill_window(const LevelParams &p, int pid, int x0, int y0, int cur,
-                                         float af, int pcur) {
+__device__ __noinline__ void fill_window(const LevelParams &p, int pid, int x0, int y0, int rows,
+                                         int cur, float af, int pcur) {
     const PatchDevice &P = p.table[pid];
     const int nx = P.nx, ny = P.ny;
-    const int ylast = (y0 + p.rows < ny ? y0 + p.rows : ny) - 1;
+    const int ylast = (y0 + rows < ny ? y0 + rows : ny) - 1;
     const int cx0 = x0 - 2 > 0 ? x0 - 2 : 0, cx1 = x0 + 29 < nx - 1 ? x0 + 29 : nx - 1;
     const int ry0 = y0 - 2 > 0 ? y0 - 2 : 0, ry1 = ylast + 2 < ny - 1 ? ylast + 2 : ny - 1;
     if (cx0 >= 2 && cx1 < nx - 2 && ry0 >= 2 && ry1 < ny - 2) return;   // no ring cell
@@ -336,41 +344,44 @@ __global__ void __launch_bounds__(strip::kThreads, 4) level_strip_kernel(LevelPa
         __syncthreads();
     }
     const int cur = s_cur;
-    const int wpb = blockDim.x >> 5;
     float smax = 0.f;
     bool bad = false;
-    // warp-uniform walk of the level's strip list
-    for (int u = blockIdx.x * wpb + (threadIdx.x >> 5); u < p.nunits; u += gridDim.x * wpb) {
+    // Warps take the level's strips from the clock's counter, then its
+    // refluxing tasks (they start as warps run out of strips; the clock is
+    // not advanced before every block has finished them).
+    const int ntasks = (p.rf.nfine + 7) / 8 + (p.rf.ncoarse + 7) / 8;
+    const int lane = threadIdx.x & 31;
+    for (;;) {   // warp-uniform
+        int u = 0;
+        if (lane == 0) u = (int)atomicAdd(&p.clk->work, 1u);
+        u = __shfl_sync(0xffffffffu, u, 0);
+        if (u >= p.nunits) {
+            if (u >= p.nunits + ntasks) break;
+            level_reflux_task(p, u - p.nunits, cur, s_nu[0], s_nu[1],
+                              reflux::coming_dt(p.clk, p.t_end), p.fill_on ? s_af : 0.f,
+                              p.fill_on ? s_pcur : 0);
+            continue;
+        }
         const int4 t = p.units[u];
         const PatchDevice &P = p.table[t.x];
         strip::View v;
         v.q0 = P.q[cur][0]; v.q1 = P.q[cur][1]; v.q2 = P.q[cur][2]; v.hb = P.hb;
         v.o0 = P.q[cur ^ 1][0]; v.o1 = P.q[cur ^ 1][1]; v.o2 = P.q[cur ^ 1][2];
         v.nx = P.nx; v.ny = P.ny; v.rdx = P.rdx; v.rdy = P.rdy; v.bc = P.bc;
+        const int rows = strip_rows(v.ny, p.rows);
         if (p.fill_on) {
-            fill_window(p, t.x, t.y, t.z, cur, s_af, s_pcur);
+            fill_window(p, t.x, t.y, t.z, rows, cur, s_af, s_pcur);
             __threadfence_block();
             __syncwarp();   // the window's writes before the strip's loads
         }
         // A strip that has had waves keeps them: it skips the quiet scan (the
         // hint only; the scan alone decides that a strip is quiet).
         if (t.w == 0) {
-            if (strip::quiet_unit<false>(v, nullptr, 0, t.y, t.z, p.rows, p.g, smax)) continue;
-            if ((threadIdx.x & 31) == 0) p.units[u].w = 1;
+            if (strip::quiet_unit<false>(v, nullptr, 0, t.y, t.z, rows, p.g, smax)) continue;
+            if (lane == 0) p.units[u].w = 1;
         }
-        strip::strip_unit<ORD, 1>(v, t.y, t.z, p.rows, s_nu[0], s_nu[1], p.g,
-                               ring[threadIdx.x >> 5], smax, bad);
-    }
-    if (p.rf.nfine + p.rf.ncoarse > 0) {
-        // the warps with one strip fewer start on the refluxing tasks; the
-        // clock is not advanced before every block has finished them
-        const int total = gridDim.x * wpb, gw = blockIdx.x * wpb + (threadIdx.x >> 5);
-        const int ntasks = (p.rf.nfine + 7) / 8 + (p.rf.ncoarse + 7) / 8;
-        const int rem = p.nunits % total;
-        const double dt_now = reflux::coming_dt(p.clk, p.t_end);
-        for (int t = (gw + total - rem) % total; t < ntasks; t += total)
-            level_reflux_task(p, t, cur, s_nu[0], s_nu[1], dt_now, p.fill_on ? s_af : 0.f,
-                              p.fill_on ? s_pcur : 0);
+        strip::strip_unit<ORD, 1>(v, t.y, t.z, rows, s_nu[0], s_nu[1], p.g,
+                                  ring[threadIdx.x >> 5], smax, bad);
     }
     if (bad) atomicOr(p.err, ERR_UNSTABLE);
     fwave::finish_step<strip::kThreads>(p.clk, p.partial, p.nblocks, p.cfl, smax, red,
@@ -388,7 +399,8 @@ __global__ void level_smax_kernel(LevelParams p, double *smax) {
     for (int k = blockIdx.x; k < p.nunits; k += gridDim.x) {
         const int4 t = p.units[k];
         const PatchDevice &P = p.table[t.x];
-        for (int c = threadIdx.x; c < strip::kOut * p.rows; c += blockDim.x) {
+        const int rows = strip_rows(P.ny, p.rows);
+        for (int c = threadIdx.x; c < strip::kOut * rows; c += blockDim.x) {
             const int i = t.y + c % strip::kOut, j = t.z + c / strip::kOut;
             if (i >= P.nx || j >= P.ny) continue;
             const size_t o = (size_t)j * P.nx + i;
@@ -437,15 +449,20 @@ unsigned ew_blocks(size_t n) {
     return (unsigned)(b > 4096 ? 4096 : (b < 1 ? 1 : b));
 }
 
+// Strip lists of a level: heights 16, 32 and the default's.
+constexpr int kHeights = 3, kDefault = 2;
+constexpr int kMinRows = 4, kMaxRows = 36;   // bounds of the default height
+
 struct Level {
-    int npatches = 0, nunits16 = 0, nunits32 = 0;
+    int npatches = 0;
     long long ncells = 0;
     double dx = 0, dy = 0;
-    int4 *units16 = nullptr, *units32 = nullptr;
+    int4 *units[kHeights] = {nullptr, nullptr, nullptr};   // strip lists by height
+    int nunits[kHeights] = {0, 0, 0}, height[kHeights] = {16, 32, 0};
     DevClock *clk = nullptr;
     double *partial = nullptr;
     double *smax = nullptr;
-    int rows = 0;   // requested strip height (16 or 32), 0 = default 32
+    int rows = 0;   // requested strip height (16 or 32), 0 = default
     bool started = false;
 };
 
@@ -524,19 +541,65 @@ int check_patches(int n, const swa_patch_desc *p, const swa_grid_desc *c) {
     return SWA_OK;
 }
 
-void strips_of(const swa_patch_desc &p, int k, int rows, std::vector<int4> &out) {
-    for (int j0 = 0; j0 < p.ny; j0 += rows)
-        for (int i0 = 0; i0 < p.nx; i0 += strip::kOut) out.push_back(make_int4(k, i0, j0, 0));
+long long strip_count(const swa_patch_desc &p, int rows) {
+    const int h = strip_rows(p.ny, rows);
+    return (long long)((p.nx + strip::kOut - 1) / strip::kOut) * ((p.ny + h - 1) / h);
+}
+
+// The strips of every patch of level l, at most `rows` rows high, higher
+// ones first (the last strips a launch takes are then short ones).
+std::vector<int4> strips_of(int n, const swa_patch_desc *p, int l, int rows) {
+    std::vector<int> ids;
+    for (int k = 0; k < n; k++)
+        if (p[k].level == l) ids.push_back(k);
+    std::stable_sort(ids.begin(), ids.end(), [&](int a, int b) {
+        return strip_rows(p[a].ny, rows) > strip_rows(p[b].ny, rows);
+    });
+    std::vector<int4> out;
+    for (int k : ids) {
+        const int h = strip_rows(p[k].ny, rows);
+        for (int j0 = 0; j0 < p[k].ny; j0 += h)
+            for (int i0 = 0; i0 < p[k].nx; i0 += strip::kOut) out.push_back(make_int4(k, i0, j0, 0));
+    }
+    return out;
+}
+
+// The default strip height of level l: the lowest (at least kMinRows) whose
+// strips are no more than k times the resident warps, for the smallest k
+// that needs no more than kMaxRows rows (the single grid's rule: a level of
+// few strips is latency-bound, one of many wants them high and a whole
+// number of rounds).
+// Measured on three levels of 160 patches with sides 16 to 256 (2.9 M cells
+// each), us per step, 32 rows by block index / this rule from the counter:
+// 65.6, 64.0, 63.9 / 55.2, 51.1, 50.2; 64 patches of 132^2: about 40 / 28.
+int default_rows(int n, const swa_patch_desc *p, int l) {
+    const long long warps = (long long)occupancy_blocks() * (strip::kThreads / 32);
+    auto count = [&](int rows) {
+        long long c = 0;
+        for (int k = 0; k < n; k++)
+            if (p[k].level == l) c += strip_count(p[k], rows);
+        return c;
+    };
+    const long long rounds = (count(kMaxRows) + warps - 1) / warps;
+    int lo = kMinRows, hi = kMaxRows;
+    while (lo < hi) {   // the count falls with the height
+        const int mid = (lo + hi) / 2;
+        if (count(mid) <= rounds * warps) hi = mid;
+        else lo = mid + 1;
+    }
+    return lo;
 }
 
 void layout(int n, const swa_patch_desc *p, Carve &c, swa_patchset *ps) {
     size_t maxn = 0;
-    std::vector<int4> t16[SWA_MAX_LEVELS + 1], t32[SWA_MAX_LEVELS + 1];
+    size_t count[SWA_MAX_LEVELS + 1][kHeights] = {};
     for (int k = 0; k < n; k++) {
         const size_t nn = (size_t)p[k].nx * p[k].ny;
         if (nn > maxn) maxn = nn;
-        strips_of(p[k], k, 16, t16[p[k].level]);
-        strips_of(p[k], k, 32, t32[p[k].level]);
+        size_t *c = count[p[k].level];
+        c[0] += strip_count(p[k], 16);
+        c[1] += strip_count(p[k], 32);
+        c[kDefault] += strip_count(p[k], kMinRows);   // at most
     }
     PatchDevice *table = (PatchDevice *)c.take(sizeof(PatchDevice) * n);
     double *staging = (double *)c.take(maxn * 8);
@@ -561,16 +624,15 @@ void layout(int n, const swa_patch_desc *p, Carve &c, swa_patchset *ps) {
         }
     }
     for (int l = 1; l <= SWA_MAX_LEVELS; l++) {
-        int4 *a = (int4 *)c.take(sizeof(int4) * (t16[l].size() + 1));
-        int4 *b = (int4 *)c.take(sizeof(int4) * (t32[l].size() + 1));
+        int4 *units[kHeights];
+        for (int h = 0; h < kHeights; h++) units[h] = (int4 *)c.take(sizeof(int4) * (count[l][h] + 1));
         DevClock *clk = (DevClock *)c.take(sizeof(DevClock));
         double *part = (double *)c.take(8 * kMaxBlocks);
         double *smax = (double *)c.take(8);
         if (ps) {
             Level &L = ps->lev[l];
-            L.units16 = a; L.units32 = b; L.clk = clk; L.partial = part; L.smax = smax;
-            L.nunits16 = (int)t16[l].size();
-            L.nunits32 = (int)t32[l].size();
+            for (int h = 0; h < kHeights; h++) L.units[h] = units[h];
+            L.clk = clk; L.partial = part; L.smax = smax;
         }
     }
 }
@@ -581,13 +643,10 @@ static LevelParams level_params(const swa_patchset *ps, int l, double t_end) {
     const Level &L = ps->lev[l];
     LevelParams p{};
     p.table = ps->table;
-    // default: 16-row strips when a level has few enough of them for every
-    // resident warp to take at most one (a latency-bound level, where
-    // shorter strips shorten the critical path), 32 otherwise
-    const int auto_rows = L.nunits16 <= occupancy_blocks() * (strip::kThreads / 32) ? 16 : 32;
-    p.rows = L.rows == 16 ? 16 : (L.rows == 32 ? 32 : auto_rows);
-    p.units = p.rows == 16 ? L.units16 : L.units32;
-    p.nunits = p.rows == 16 ? L.nunits16 : L.nunits32;
+    const int h = L.rows == 16 ? 0 : (L.rows == 32 ? 1 : kDefault);
+    p.rows = L.height[h];
+    p.units = L.units[h];
+    p.nunits = L.nunits[h];
     p.clk = L.clk;
     p.partial = L.partial;
     p.t_end = t_end;
@@ -619,11 +678,10 @@ static int level_launch(swa_patchset *ps, int level, int nsteps, double t_end,
     p.nblocks = occupancy_blocks();
     if (p.nblocks > need) p.nblocks = need;
     for (int s = 0; s < nsteps; s++)
-        if (p.order == 2)
-            level_strip_kernel<2><<<p.nblocks, strip::kThreads, 0, st>>>(p);
-        else
-            level_strip_kernel<1><<<p.nblocks, strip::kThreads, 0, st>>>(p);
-    return cuda_check(cudaGetLastError(), "level_strip_kernel");
+        TRY(cuda_check(launch_chained(p.order == 2 ? level_strip_kernel<2> : level_strip_kernel<1>,
+                                      p.nblocks, strip::kThreads, 0, st, p),
+                       "level_strip_kernel"));
+    return SWA_OK;
 }
 
 extern "C" {
@@ -655,24 +713,25 @@ int swa_create_patches(int n, const swa_patch_desc *patches, const double *const
     cudaStream_t st = (cudaStream_t)stream;
     int rc = cuda_check(cudaMemsetAsync(ws, 0, need - 256, st), "workspace clear");
     // per-level bookkeeping and strip lists
-    std::vector<int4> t16[SWA_MAX_LEVELS + 1], t32[SWA_MAX_LEVELS + 1];
+    std::vector<int4> lists[SWA_MAX_LEVELS + 1][kHeights];
     for (int k = 0; k < n; k++) {
         Level &L = ps->lev[patches[k].level];
         L.npatches++;
         L.ncells += (long long)patches[k].nx * patches[k].ny;
         L.dx = patches[k].dx;
         L.dy = patches[k].dy;
-        strips_of(patches[k], k, 16, t16[patches[k].level]);
-        strips_of(patches[k], k, 32, t32[patches[k].level]);
     }
     for (int l = 1; l <= SWA_MAX_LEVELS && rc == SWA_OK; l++) {
         Level &L = ps->lev[l];
         if (L.npatches == 0) continue;
-        rc = cuda_check(cudaMemcpyAsync(L.units16, t16[l].data(), sizeof(int4) * t16[l].size(),
-                                        cudaMemcpyHostToDevice, st), "strip list upload");
-        if (rc == SWA_OK)
-            rc = cuda_check(cudaMemcpyAsync(L.units32, t32[l].data(), sizeof(int4) * t32[l].size(),
+        L.height[kDefault] = default_rows(n, patches, l);
+        for (int h = 0; h < kHeights && rc == SWA_OK; h++) {
+            std::vector<int4> &u = lists[l][h];
+            u = strips_of(n, patches, l, L.height[h]);
+            L.nunits[h] = (int)u.size();
+            rc = cuda_check(cudaMemcpyAsync(L.units[h], u.data(), sizeof(int4) * u.size(),
                                             cudaMemcpyHostToDevice, st), "strip list upload");
+        }
     }
     if (rc == SWA_OK)
         rc = cuda_check(cudaMemcpyAsync(ps->table, ps->host_table.data(),
@@ -734,10 +793,8 @@ int swa_patches_start_level(swa_patchset *ps, int level, double t, void *stream)
     cudaStream_t st = (cudaStream_t)stream;
     LevelParams p = level_params(ps, level, 0.0);
     TRY(cuda_check(cudaMemsetAsync(L.smax, 0, 8, st), "smax clear"));
-    if (L.nunits16 > 0)
-        clear_hint_kernel<<<(L.nunits16 + 255) / 256, 256, 0, st>>>(L.units16, L.nunits16);
-    if (L.nunits32 > 0)
-        clear_hint_kernel<<<(L.nunits32 + 255) / 256, 256, 0, st>>>(L.units32, L.nunits32);
+    for (int h = 0; h < kHeights; h++)
+        clear_hint_kernel<<<(L.nunits[h] + 255) / 256, 256, 0, st>>>(L.units[h], L.nunits[h]);
     TRY(cuda_check(cudaGetLastError(), "clear_hint_kernel"));
     int blocks = p.nunits < 2048 ? p.nunits : 2048;
     level_smax_kernel<<<blocks, 256, 0, st>>>(p, L.smax);

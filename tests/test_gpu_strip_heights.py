@@ -68,3 +68,38 @@ def test_gauge_groups_equal_samples(S, n):
     assert S.swa_grid_gauge_rows(g2.h) == steps
     assert torch.equal(series, ref[:cap])
     assert np.array_equal(times.cpu().numpy(), np.array(tref[:cap]))
+
+
+@pytest.mark.parametrize("count,side", [(1, 2), (3, 37), (40, 33), (30, 260)])
+@pytest.mark.parametrize("order", [1, 2])
+def test_default_patch_strips_equal_fixed_ones(S, count, side, order):
+    """A level's default strips (4 to 36 rows, bands of equal height, taken
+    from a counter) give the bits of the 16- and 32-row ones."""
+    rng = np.random.default_rng(count)
+    pats, fields = [], []
+    for k in range(count):
+        nx, ny = (2, 2) if side == 2 else (int(rng.integers(2, side)), int(rng.integers(2, side)))
+        pats.append((1, 0.0, 0.0, nx, ny, 1e3, 1e3))
+        n = nx * ny
+        B = -rng.uniform(50.0, 4000.0) * np.ones(n)
+        eta = rng.uniform(-1, 1, n) if k % 3 else np.zeros(n)
+        hu = rng.uniform(-5, 5, n) if k % 3 else np.zeros(n)
+        fields.append((B, eta, hu, -hu))
+    common = S.make_desc(2, 2, 2, 0.0, 0.0, 1e3, 1e3, precision=S.SWA_FP32, order=order)
+    ref = None
+    for rows in (0, 16, 32):
+        ps = S.PatchSet(pats, [f[0] for f in fields], common)
+        for k, f in enumerate(fields):
+            ps.set_state(k, *f[1:])
+        S.swa_patches_set_tile_rows(ps.h, 1, rows)
+        ps.start(1, 0.0)
+        ps.step(1, 9)
+        got = [ps.get_state(k) for k in range(count)]
+        t = ps.time(1)
+        if ref is None:
+            ref, t_ref = got, t
+        assert t == t_ref
+        for a, b in zip(ref, got):
+            for key in a:
+                assert np.array_equal(a[key], b[key])
+    assert S.swa_sync_status() == 0
