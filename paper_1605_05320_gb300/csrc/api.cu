@@ -111,16 +111,47 @@ __global__ void conv_in_kernel(const double *src, R *dst, const double *Bd, int 
     }
 }
 
-// mode for conv_out: 0 dst = src; 1 dst = src + bath (double B or float hbar)
+// A grid's state as FP64 arrays (any may be null): the current buffer is read
+// from the device clock, so nothing waits for it.
 template <typename R>
-__global__ void conv_out_kernel(const R *src, const R *bath, double *dst, int mode,
-                                size_t n) {
+struct StateOut {
+    const DevClock *clk;
+    const R *q[2][3];
+    const R *bath;
+    double *h, *hu, *hv, *eta;
+    int two_d;
+};
+template <typename R>
+__global__ void state_out_kernel(StateOut<R> p, size_t n) {
+    const int cur = p.clk->cur;
     for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
          k += (size_t)gridDim.x * blockDim.x) {
-        double v = (double)src[k];
-        if (mode == 1) v = v + (double)bath[k];
-        dst[k] = v;
+        const double a = (double)p.q[cur][0][k];
+        if (sizeof(R) == 8) {   // h; eta = h + B
+            if (p.h) p.h[k] = a;
+            if (p.eta) p.eta[k] = a + (double)p.bath[k];
+        } else {                // eta; h = eta + hbar
+            if (p.h) p.h[k] = a + (double)p.bath[k];
+            if (p.eta) p.eta[k] = a;
+        }
+        if (p.hu) p.hu[k] = (double)p.q[cur][1][k];
+        if (p.hv) p.hv[k] = p.two_d ? (double)p.q[cur][2][k] : 0.0;
     }
+}
+
+// Up to three arrays converted in one launch, dst[c] = (D) src[c].
+template <typename S, typename D>
+struct Conv3 {
+    const S *src[3];
+    D *dst[3];
+};
+template <typename S, typename D>
+__global__ void conv3_kernel(Conv3<S, D> p, int nc, size_t n) {
+    for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
+         k += (size_t)gridDim.x * blockDim.x)
+#pragma unroll
+        for (int c = 0; c < 3; c++)
+            if (c < nc) p.dst[c][k] = (D)p.src[c][k];
 }
 
 __global__ void fill_zero_f64(double *p, size_t n) {
@@ -150,11 +181,10 @@ static int conv_in(const double *src, R *dst, const double *Bd, int mode, size_t
     return cuda_check(cudaGetLastError(), "conv_in_kernel");
 }
 
-template <typename R>
-static int conv_out(const R *src, const R *bath, double *dst, int mode, size_t n,
-                    cudaStream_t st) {
-    conv_out_kernel<R><<<ew_blocks(n), 256, 0, st>>>(src, bath, dst, mode, n);
-    return cuda_check(cudaGetLastError(), "conv_out_kernel");
+template <typename S, typename D>
+static int conv3(const Conv3<S, D> &p, int nc, size_t n, cudaStream_t st) {
+    conv3_kernel<S, D><<<ew_blocks(n), 256, 0, st>>>(p, nc, n);
+    return cuda_check(cudaGetLastError(), "conv3_kernel");
 }
 
 // ------------------------------------------------------------------- grid
@@ -294,6 +324,25 @@ static FwdParams<R> fwd_params(const swa_grid *g, double t_end) {
     return p;
 }
 
+template <typename R>
+static int state_out_as(const swa_grid *g, double *const dst[4], cudaStream_t st) {
+    StateOut<R> p{};
+    p.clk = g->clk;
+    for (int b = 0; b < 2; b++)
+        for (int k = 0; k < 3; k++) p.q[b][k] = (const R *)g->q[b][k];
+    p.bath = (const R *)g->bath;
+    p.h = dst[0]; p.hu = dst[1]; p.hv = dst[2]; p.eta = dst[3];
+    p.two_d = g->d.ndim == 2;
+    state_out_kernel<R><<<ew_blocks(g->n), 256, 0, st>>>(p, g->n);
+    return cuda_check(cudaGetLastError(), "state_out_kernel");
+}
+
+// The current state into device arrays (h, hu, hv, eta; any may be null).
+static int state_out(const swa_grid *g, double *const dst[4], cudaStream_t st) {
+    return g->d.precision == SWA_FP64 ? state_out_as<double>(g, dst, st)
+                                      : state_out_as<float>(g, dst, st);
+}
+
 extern "C" {
 
 const char *swa_version(void) { return "swadj 0.1 (sm_103a)"; }
@@ -384,32 +433,33 @@ static int set_state_impl(swa_grid *g, const double *eta, const double *hu, cons
     if (g->d.ndim == 2 && !hv) return set_error(SWA_EINVAL, "hv required for 2D grids");
     if (where != SWA_HOST && where != SWA_DEVICE) return set_error(SWA_EINVAL, "bad where");
     cudaStream_t st = S(stream);
-    const double *src[3] = {eta, hu, hv};
-    const int nf = g->d.ndim == 2 ? 3 : 2;
-    for (int k = 0; k < nf; k++) {
-        const double *s = src[k];
-        if (where == SWA_HOST) {
-            TRY(cuda_check(cudaMemcpyAsync(g->staging, s, g->n * 8, cudaMemcpyHostToDevice, st),
+    const StateSrc dev{eta, hu, hv}, *src = &dev;
+    if (where == SWA_HOST) {   // one staging array: converted field by field
+        const double *f[3] = {eta, hu, hv};
+        const int nf = g->d.ndim == 2 ? 3 : 2;
+        for (int k = 0; k < nf; k++) {
+            TRY(cuda_check(cudaMemcpyAsync(g->staging, f[k], g->n * 8, cudaMemcpyHostToDevice, st),
                            "state upload"));
-            s = g->staging;
+            if (g->d.precision == SWA_FP64)
+                TRY(conv_in<double>(g->staging, (double *)g->q[0][k], g->Bd, k == 0 ? 1 : 0, g->n,
+                                    st));
+            else
+                TRY(conv_in<float>(g->staging, (float *)g->q[0][k], nullptr, 0, g->n, st));
         }
-        if (g->d.precision == SWA_FP64)
-            TRY(conv_in<double>(s, (double *)g->q[0][k], g->Bd, k == 0 ? 1 : 0, g->n, st));
-        else
-            TRY(conv_in<float>(s, (float *)g->q[0][k], nullptr, 0, g->n, st));
+        if (nf == 2)
+            TRY(cuda_check(cudaMemsetAsync(g->q[0][2], 0, g->n * g->esz, st), "hv clear"));
+        src = nullptr;
     }
-    if (nf == 2) {
-        TRY(cuda_check(cudaMemsetAsync(g->q[0][2], 0, g->n * g->esz, st), "hv clear"));
-    }
-    TRY(cuda_check(cudaMemsetAsync(g->q[1][2], 0, g->n * g->esz, st), "hv clear"));
+    if (g->d.ndim == 1)   // the 1D steps do not write hv
+        TRY(cuda_check(cudaMemsetAsync(g->q[1][2], 0, g->n * g->esz, st), "hv clear"));
     if (g->d.precision == SWA_FP64) {
         FwdParams<double> p = fwd_params<double>(g, 0.0);
         if (!check) p.err = nullptr;
-        TRY(fwd_launch_clock_init<double>(p, t, st));
+        TRY(fwd_launch_clock_init<double>(p, t, src, st));
     } else {
         FwdParams<float> p = fwd_params<float>(g, 0.0);
         if (!check) p.err = nullptr;
-        TRY(fwd_launch_clock_init<float>(p, t, st));
+        TRY(fwd_launch_clock_init<float>(p, t, src, st));
     }
     g->state_set = 1;
     return SWA_OK;
@@ -425,36 +475,16 @@ int swa_get_state(swa_grid *g, double *h, double *hu, double *hv, double *eta, i
     if (!g) return set_error(SWA_EINVAL, "null grid");
     if (where != SWA_HOST && where != SWA_DEVICE) return set_error(SWA_EINVAL, "bad where");
     cudaStream_t st = S(stream);
-    DevClock clk;
-    TRY(cuda_check(cudaMemcpyAsync(&clk, g->clk, sizeof(clk), cudaMemcpyDeviceToHost, st),
-                   "clock read"));
-    TRY(cuda_check(cudaStreamSynchronize(st), "clock read"));
-    const int cur = clk.cur;
     double *dst[4] = {h, hu, hv, eta};
-    for (int k = 0; k < 4; k++) {
+    if (where == SWA_DEVICE) return state_out(g, dst, st);
+    for (int k = 0; k < 4; k++) {   // one staging array: field by field
         if (!dst[k]) continue;
-        if (k == 2 && g->d.ndim == 1) {
-            if (where == SWA_HOST) memset(dst[k], 0, g->n * 8);
-            else TRY(cuda_check(cudaMemsetAsync(dst[k], 0, g->n * 8, st), "hv clear"));
-            continue;
-        }
-        double *d = where == SWA_HOST ? g->staging : dst[k];
-        const int field = k == 3 ? 0 : k;
-        int mode = 0;
-        if (g->d.precision == SWA_FP64) {
-            mode = (k == 3) ? 1 : 0;  // eta = h + B
-            TRY(conv_out<double>((const double *)g->q[cur][field], (const double *)g->bath, d,
-                                 mode, g->n, st));
-        } else {
-            mode = (k == 0) ? 1 : 0;  // h = eta + hbar
-            TRY(conv_out<float>((const float *)g->q[cur][field], (const float *)g->bath, d,
-                                mode, g->n, st));
-        }
-        if (where == SWA_HOST) {
-            TRY(cuda_check(cudaMemcpyAsync(dst[k], g->staging, g->n * 8,
-                                           cudaMemcpyDeviceToHost, st), "state download"));
-            TRY(cuda_check(cudaStreamSynchronize(st), "state download"));
-        }
+        double *one[4] = {nullptr, nullptr, nullptr, nullptr};
+        one[k] = g->staging;
+        TRY(state_out(g, one, st));
+        TRY(cuda_check(cudaMemcpyAsync(dst[k], g->staging, g->n * 8, cudaMemcpyDeviceToHost, st),
+                       "state download"));
+        TRY(cuda_check(cudaStreamSynchronize(st), "state download"));
     }
     return SWA_OK;
 }
@@ -604,6 +634,35 @@ static AdjParams<R> adj_params(const swa_adjoint *a) {
     p.umap = a->umap;
     p.umap_n = a->umap_n;
     return p;
+}
+
+// Components first .. first + nc - 1 of the state to or from nc x n FP64
+// values on the device (buffer cur, or buffer 0 when set).
+template <typename R>
+static int adj_out_as(const swa_adjoint *a, int first, int nc, double *q, cudaStream_t st) {
+    Conv3<R, double> p{};
+    for (int c = 0; c < nc; c++) {
+        p.src[c] = (const R *)a->q[a->cur][first + c];
+        p.dst[c] = q + (size_t)c * a->n;
+    }
+    return conv3(p, nc, a->n, st);
+}
+static int adj_out(const swa_adjoint *a, int first, int nc, double *q, cudaStream_t st) {
+    return a->d.precision == SWA_FP64 ? adj_out_as<double>(a, first, nc, q, st)
+                                      : adj_out_as<float>(a, first, nc, q, st);
+}
+template <typename R>
+static int adj_in_as(const swa_adjoint *a, int first, int nc, const double *phi, cudaStream_t st) {
+    Conv3<double, R> p{};
+    for (int c = 0; c < nc; c++) {
+        p.src[c] = phi + (size_t)c * a->n;
+        p.dst[c] = (R *)a->q[0][first + c];
+    }
+    return conv3(p, nc, a->n, st);
+}
+static int adj_in(const swa_adjoint *a, int first, int nc, const double *phi, cudaStream_t st) {
+    return a->d.precision == SWA_FP64 ? adj_in_as<double>(a, first, nc, phi, st)
+                                      : adj_in_as<float>(a, first, nc, phi, st);
 }
 
 // ---------------------------------------------------------------- snapshots
@@ -827,17 +886,12 @@ int swa_adjoint_set_steps_per_pass(swa_adjoint *a, int k) {
 int swa_get_adjoint_state(swa_adjoint *a, double *q, int where, void *stream) {
     if (!a || !q) return set_error(SWA_EINVAL, "null argument");
     cudaStream_t st = S(stream);
-    for (int k = 0; k < a->nc; k++) {
-        double *d = where == SWA_HOST ? a->staging : q + (size_t)k * a->n;
-        if (a->d.precision == SWA_FP64)
-            TRY(conv_out<double>((const double *)a->q[a->cur][k], nullptr, d, 0, a->n, st));
-        else
-            TRY(conv_out<float>((const float *)a->q[a->cur][k], nullptr, d, 0, a->n, st));
-        if (where == SWA_HOST) {
-            TRY(cuda_check(cudaMemcpyAsync(q + (size_t)k * a->n, a->staging, a->n * 8,
-                                           cudaMemcpyDeviceToHost, st), "adjoint download"));
-            TRY(cuda_check(cudaStreamSynchronize(st), "adjoint download"));
-        }
+    if (where != SWA_HOST) return adj_out(a, 0, a->nc, q, st);
+    for (int k = 0; k < a->nc; k++) {   // one staging array: component by component
+        TRY(adj_out(a, k, 1, a->staging, st));
+        TRY(cuda_check(cudaMemcpyAsync(q + (size_t)k * a->n, a->staging, a->n * 8,
+                                       cudaMemcpyDeviceToHost, st), "adjoint download"));
+        TRY(cuda_check(cudaStreamSynchronize(st), "adjoint download"));
     }
     return SWA_OK;
 }
@@ -846,17 +900,14 @@ int swa_set_adjoint_state(swa_adjoint *a, const double *phi, int where, void *st
     if (!a || !phi) return set_error(SWA_EINVAL, "null argument");
     if (where != SWA_HOST && where != SWA_DEVICE) return set_error(SWA_EINVAL, "bad where");
     cudaStream_t st = S(stream);
-    for (int k = 0; k < a->nc; k++) {
-        const double *src = phi + (size_t)k * a->n;
-        if (where == SWA_HOST) {
-            TRY(cuda_check(cudaMemcpyAsync(a->staging, src, a->n * 8, cudaMemcpyHostToDevice, st),
-                           "phi upload"));
-            src = a->staging;
+    if (where == SWA_DEVICE) {
+        TRY(adj_in(a, 0, a->nc, phi, st));
+    } else {
+        for (int k = 0; k < a->nc; k++) {   // one staging array: component by component
+            TRY(cuda_check(cudaMemcpyAsync(a->staging, phi + (size_t)k * a->n, a->n * 8,
+                                           cudaMemcpyHostToDevice, st), "phi upload"));
+            TRY(adj_in(a, k, 1, a->staging, st));
         }
-        if (a->d.precision == SWA_FP64)
-            TRY(conv_in<double>(src, (double *)a->q[0][k], nullptr, 0, a->n, st));
-        else
-            TRY(conv_in<float>(src, (float *)a->q[0][k], nullptr, 0, a->n, st));
     }
     if (a->umap)   // a new state: no unit has had a nonzero value yet
         TRY(cuda_check(cudaMemsetAsync(a->umap, 0, (size_t)a->umap_n, st), "unit map clear"));

@@ -31,6 +31,11 @@ struct FwdParams {
     R dry_tol;         // a cell with h <= dry_tol is dry
 };
 
+// FP64 arrays on the device that a state is set from (hv unused in 1D).
+struct StateSrc {
+    const double *eta, *hu, *hv;
+};
+
 template <typename R>
 int fwd_launch_step(const FwdParams<R> &p, cudaStream_t st);
 // rest CFL table of the FP32 2D grid step (floats, and the kernel filling it)
@@ -39,8 +44,9 @@ int fwd_f32_unit_map_bytes(int nx, int ny);
 int fwd_f32_rest_table(const FwdParams<float> &p, float *tab, cudaStream_t st);
 template <typename R>
 int fwd_step_blocks(const FwdParams<R> &p);
+// First clock of the state in buffer 0; src: set that buffer from it first.
 template <typename R>
-int fwd_launch_clock_init(const FwdParams<R> &p, double t0, cudaStream_t st);
+int fwd_launch_clock_init(const FwdParams<R> &p, double t0, const StateSrc *src, cudaStream_t st);
 template <> int fwd_launch_step<double>(const FwdParams<double> &, cudaStream_t);
 template <> int fwd_launch_step<float>(const FwdParams<float> &, cudaStream_t);
 template <> int fwd_step_blocks<double>(const FwdParams<double> &);
@@ -63,7 +69,9 @@ template <> int fwd_launch_wd<double>(const FwdParams<double> &, cudaStream_t);
 template <> int fwd_launch_wd<float>(const FwdParams<float> &, cudaStream_t);
 template <> int fwd_wd_blocks<double>(const FwdParams<double> &);
 template <> int fwd_wd_blocks<float>(const FwdParams<float> &);
-template <> int fwd_launch_clock_init<double>(const FwdParams<double> &, double, cudaStream_t);
-template <> int fwd_launch_clock_init<float>(const FwdParams<float> &, double, cudaStream_t);
+template <> int fwd_launch_clock_init<double>(const FwdParams<double> &, double,
+                                              const StateSrc *, cudaStream_t);
+template <> int fwd_launch_clock_init<float>(const FwdParams<float> &, double,
+                                             const StateSrc *, cudaStream_t);
 
 }  // namespace swadj

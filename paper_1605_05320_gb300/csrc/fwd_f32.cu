@@ -300,11 +300,15 @@ int fwd_ctu_blocks<float>(const FwdParams<float> &p) {
 }
 
 template <>
-int fwd_launch_clock_init<float>(const FwdParams<float> &p, double t0, cudaStream_t st) {
+int fwd_launch_clock_init<float>(const FwdParams<float> &p, double t0, const StateSrc *src,
+                                 cudaStream_t st) {
     const size_t n = (size_t)p.nx * p.ny;
     int blocks = (int)((n + 255) / 256);
     if (blocks > kInitBlocks) blocks = kInitBlocks;
-    clock_init_kernel<float, true><<<blocks, 256, 0, st>>>(p, t0);
+    if (src)
+        clock_init_kernel<float, true, true><<<blocks, 256, 0, st>>>(p, t0, *src);
+    else
+        clock_init_kernel<float, true, false><<<blocks, 256, 0, st>>>(p, t0, StateSrc{});
     return swadj_host::cuda_check(cudaGetLastError(), "clock_init_kernel<float>");
 }
 

@@ -101,11 +101,15 @@ int fwd_ctu_blocks<double>(const FwdParams<double> &p) {
 }
 
 template <>
-int fwd_launch_clock_init<double>(const FwdParams<double> &p, double t0, cudaStream_t st) {
+int fwd_launch_clock_init<double>(const FwdParams<double> &p, double t0, const StateSrc *src,
+                                  cudaStream_t st) {
     const size_t n = (size_t)p.nx * p.ny;
     int blocks = (int)((n + 255) / 256);
     if (blocks > kInitBlocks) blocks = kInitBlocks;
-    clock_init_kernel<double, false><<<blocks, 256, 0, st>>>(p, t0);
+    if (src)
+        clock_init_kernel<double, false, true><<<blocks, 256, 0, st>>>(p, t0, *src);
+    else
+        clock_init_kernel<double, false, false><<<blocks, 256, 0, st>>>(p, t0, StateSrc{});
     return swadj_host::cuda_check(cudaGetLastError(), "clock_init_kernel<double>");
 }
 

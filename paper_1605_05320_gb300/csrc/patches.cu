@@ -388,19 +388,29 @@ __global__ void __launch_bounds__(strip::kThreads, 4) level_strip_kernel(LevelPa
                                         &am_last, t_now, dt, s_cur);
 }
 
-__device__ __forceinline__ void atomic_max_nonneg(double *a, double v) {
-    atomicMax((unsigned long long *)a, (unsigned long long)__double_as_longlong(v));
-}
-
-// CFL maximum of buffer 0 of every patch of the level (same per-cell rule as
-// the step's fused reduction), into *smax.
-__global__ void level_smax_kernel(LevelParams p, double *smax) {
+// Starts a level's clock at t0: clears the strips' hints (no strip of the new
+// state has had waves yet) and reduces the CFL maximum over buffer 0 of every
+// patch (the step's per-cell rule).
+struct StartParams {
+    LevelParams p;
+    int4 *units[3];
+    int nunits[3];
+    double t0;
+};
+__global__ void __launch_bounds__(256) level_start_kernel(StartParams q) {
+    __shared__ float red[8];
+    __shared__ int am_last;
+    const LevelParams &p = q.p;
+    const int tid = threadIdx.x;
+    for (int h = 0; h < 3; h++)
+        for (int k = blockIdx.x * 256 + tid; k < q.nunits[h]; k += gridDim.x * 256)
+            q.units[h][k].w = 0;
     float m = 0.f;
     for (int k = blockIdx.x; k < p.nunits; k += gridDim.x) {
         const int4 t = p.units[k];
         const PatchDevice &P = p.table[t.x];
         const int rows = strip_rows(P.ny, p.rows);
-        for (int c = threadIdx.x; c < strip::kOut * rows; c += blockDim.x) {
+        for (int c = tid; c < strip::kOut * rows; c += 256) {
             const int i = t.y + c % strip::kOut, j = t.z + c / strip::kOut;
             if (i >= P.nx || j >= P.ny) continue;
             const size_t o = (size_t)j * P.nx + i;
@@ -411,17 +421,63 @@ __global__ void level_smax_kernel(LevelParams p, double *smax) {
         }
     }
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomic_max_nonneg(smax, (double)m);
+    if ((tid & 31) == 0) red[tid >> 5] = m;
+    __syncthreads();
+    float *partial = reinterpret_cast<float *>(p.partial);
+    if (tid == 0) {
+        for (int k = 1; k < 8; k++) m = fmaxf(m, red[k]);
+        partial[blockIdx.x] = m;
+        __threadfence();
+        am_last = atomicAdd(&p.clk->ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!am_last) return;
+    __threadfence();
+    m = 0.f;
+    for (int k = tid; k < (int)gridDim.x; k += 256) m = fmaxf(m, __ldcg(partial + k));
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((tid & 31) == 0) red[tid >> 5] = m;
+    __syncthreads();
+    if (tid == 0) {
+        for (int k = 1; k < 8; k++) m = fmaxf(m, red[k]);
+        DevClock *clk = p.clk;
+        clk->t = q.t0;
+        clk->smax = (double)m;
+        clk->dt_cfl = p.cfl / (double)m;
+        clk->cur = 0;
+        clk->nsteps = 0;
+        clk->ticket = 0u;
+        clk->work = 0u;
+    }
 }
 
-__global__ void level_clock_kernel(DevClock *clk, const double *smax, double t0, double cfl) {
-    clk->t = t0;
-    clk->smax = *smax;
-    clk->dt_cfl = cfl / *smax;
-    clk->cur = 0;
-    clk->nsteps = 0;
-    clk->ticket = 0u;
-    clk->work = 0u;
+// A patch's state from FP64 arrays, and to them (any output may be null): one
+// launch for all fields, the current buffer read from the level's clock.
+__global__ void patch_set_kernel(const double *eta, const double *hu, const double *hv, float *q0,
+                                 float *q1, float *q2, size_t n) {
+    for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
+         k += (size_t)gridDim.x * blockDim.x) {
+        q0[k] = (float)eta[k];
+        q1[k] = (float)hu[k];
+        q2[k] = (float)hv[k];
+    }
+}
+
+struct PatchOut {
+    const DevClock *clk;
+    const float *q[2][3], *hb;
+    double *h, *hu, *hv, *eta;
+};
+__global__ void patch_out_kernel(PatchOut p, size_t n) {
+    const int cur = p.clk->cur;
+    for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
+         k += (size_t)gridDim.x * blockDim.x) {
+        const double a = (double)p.q[cur][0][k];
+        if (p.h) p.h[k] = a + (double)p.hb[k];
+        if (p.eta) p.eta[k] = a;
+        if (p.hu) p.hu[k] = (double)p.q[cur][1][k];
+        if (p.hv) p.hv[k] = (double)p.q[cur][2][k];
+    }
 }
 
 __global__ void to_float_kernel(const double *src, float *dst, const double *sub, int negate,
@@ -432,15 +488,6 @@ __global__ void to_float_kernel(const double *src, float *dst, const double *sub
         if (sub) v = v - sub[k];
         if (negate) v = -v;
         dst[k] = (float)v;
-    }
-}
-
-__global__ void to_double_kernel(const float *src, const float *add, double *dst, size_t n) {
-    for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
-         k += (size_t)gridDim.x * blockDim.x) {
-        double v = (double)src[k];
-        if (add) v = v + (double)add[k];
-        dst[k] = v;
     }
 }
 
@@ -461,7 +508,6 @@ struct Level {
     int nunits[kHeights] = {0, 0, 0}, height[kHeights] = {16, 32, 0};
     DevClock *clk = nullptr;
     double *partial = nullptr;
-    double *smax = nullptr;
     int rows = 0;   // requested strip height (16 or 32), 0 = default
     bool started = false;
 };
@@ -628,11 +674,10 @@ void layout(int n, const swa_patch_desc *p, Carve &c, swa_patchset *ps) {
         for (int h = 0; h < kHeights; h++) units[h] = (int4 *)c.take(sizeof(int4) * (count[l][h] + 1));
         DevClock *clk = (DevClock *)c.take(sizeof(DevClock));
         double *part = (double *)c.take(8 * kMaxBlocks);
-        double *smax = (double *)c.take(8);
         if (ps) {
             Level &L = ps->lev[l];
             for (int h = 0; h < kHeights; h++) L.units[h] = units[h];
-            L.clk = clk; L.partial = part; L.smax = smax;
+            L.clk = clk; L.partial = part;
         }
     }
 }
@@ -765,25 +810,21 @@ int swa_patches_set_state(swa_patchset *ps, int k, const double *eta, const doub
     if (where != SWA_HOST && where != SWA_DEVICE) return set_error(SWA_EINVAL, "bad where");
     cudaStream_t st = (cudaStream_t)stream;
     const size_t nn = (size_t)ps->pd[k].nx * ps->pd[k].ny;
-    const double *src[3] = {eta, hu, hv};
-    for (int m = 0; m < 3; m++) {
-        const double *s = src[m];
-        if (where == SWA_HOST) {
-            TRY(cuda_check(cudaMemcpyAsync(ps->staging, s, nn * 8, cudaMemcpyHostToDevice, st),
+    float *const *q = ps->host_table[k].q[0];
+    if (where == SWA_DEVICE) {
+        patch_set_kernel<<<ew_blocks(nn), 256, 0, st>>>(eta, hu, hv, q[0], q[1], q[2], nn);
+        TRY(cuda_check(cudaGetLastError(), "patch_set_kernel"));
+    } else {   // one staging array: converted field by field
+        const double *src[3] = {eta, hu, hv};
+        for (int m = 0; m < 3; m++) {
+            TRY(cuda_check(cudaMemcpyAsync(ps->staging, src[m], nn * 8, cudaMemcpyHostToDevice, st),
                            "state upload"));
-            s = ps->staging;
+            to_float_kernel<<<ew_blocks(nn), 256, 0, st>>>(ps->staging, q[m], nullptr, 0, nn);
+            TRY(cuda_check(cudaGetLastError(), "state convert"));
         }
-        to_float_kernel<<<ew_blocks(nn), 256, 0, st>>>(s, ps->host_table[k].q[0][m], nullptr, 0, nn);
-        TRY(cuda_check(cudaGetLastError(), "state convert"));
     }
     ps->lev[ps->pd[k].level].started = false;
     return SWA_OK;
-}
-
-// A level's new state: no strip has had waves yet (the quiet-strip hint).
-__global__ void clear_hint_kernel(int4 *u, int n) {
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
-        u[k].w = 0;
 }
 
 int swa_patches_start_level(swa_patchset *ps, int level, double t, void *stream) {
@@ -792,15 +833,12 @@ int swa_patches_start_level(swa_patchset *ps, int level, double t, void *stream)
     if (L.npatches == 0) return set_error(SWA_EINVAL, "level %d has no patches", level);
     cudaStream_t st = (cudaStream_t)stream;
     LevelParams p = level_params(ps, level, 0.0);
-    TRY(cuda_check(cudaMemsetAsync(L.smax, 0, 8, st), "smax clear"));
-    for (int h = 0; h < kHeights; h++)
-        clear_hint_kernel<<<(L.nunits[h] + 255) / 256, 256, 0, st>>>(L.units[h], L.nunits[h]);
-    TRY(cuda_check(cudaGetLastError(), "clear_hint_kernel"));
-    int blocks = p.nunits < 2048 ? p.nunits : 2048;
-    level_smax_kernel<<<blocks, 256, 0, st>>>(p, L.smax);
-    TRY(cuda_check(cudaGetLastError(), "level_smax_kernel"));
-    level_clock_kernel<<<1, 1, 0, st>>>(L.clk, L.smax, t, ps->common.cfl);
-    TRY(cuda_check(cudaGetLastError(), "level_clock_kernel"));
+    StartParams q{};
+    q.p = p;
+    for (int h = 0; h < kHeights; h++) { q.units[h] = L.units[h]; q.nunits[h] = L.nunits[h]; }
+    q.t0 = t;
+    level_start_kernel<<<p.nunits < 2048 ? p.nunits : 2048, 256, 0, st>>>(q);
+    TRY(cuda_check(cudaGetLastError(), "level_start_kernel"));
     L.started = true;
     return SWA_OK;
 }
@@ -809,25 +847,27 @@ int swa_patches_get_state(swa_patchset *ps, int k, double *h, double *hu, double
                           double *eta, int where, void *stream) {
     if (!ps || k < 0 || k >= ps->n) return set_error(SWA_EINVAL, "bad argument");
     cudaStream_t st = (cudaStream_t)stream;
-    DevClock clk;
-    TRY(cuda_check(cudaMemcpyAsync(&clk, ps->lev[ps->pd[k].level].clk, sizeof(clk),
-                                   cudaMemcpyDeviceToHost, st), "clock read"));
-    TRY(cuda_check(cudaStreamSynchronize(st), "clock read"));
-    const int cur = clk.cur;
     const size_t nn = (size_t)ps->pd[k].nx * ps->pd[k].ny;
-    double *dst[4] = {h, hu, hv, eta};
     const PatchDevice &P = ps->host_table[k];
-    for (int m = 0; m < 4; m++) {
+    PatchOut p{};
+    p.clk = ps->lev[ps->pd[k].level].clk;
+    for (int b = 0; b < 2; b++)
+        for (int m = 0; m < 3; m++) p.q[b][m] = P.q[b][m];
+    p.hb = P.hb;
+    if (where != SWA_HOST) {
+        p.h = h; p.hu = hu; p.hv = hv; p.eta = eta;
+        patch_out_kernel<<<ew_blocks(nn), 256, 0, st>>>(p, nn);
+        return cuda_check(cudaGetLastError(), "patch_out_kernel");
+    }
+    double *dst[4] = {h, hu, hv, eta}, **field[4] = {&p.h, &p.hu, &p.hv, &p.eta};
+    for (int m = 0; m < 4; m++) {   // one staging array: field by field
         if (!dst[m]) continue;
-        double *d = where == SWA_HOST ? ps->staging : dst[m];
-        const float *src = P.q[cur][m == 3 ? 0 : m];
-        to_double_kernel<<<ew_blocks(nn), 256, 0, st>>>(src, m == 0 ? P.hb : nullptr, d, nn);
-        TRY(cuda_check(cudaGetLastError(), "state convert"));
-        if (where == SWA_HOST) {
-            TRY(cuda_check(cudaMemcpyAsync(dst[m], ps->staging, nn * 8, cudaMemcpyDeviceToHost, st),
-                           "state download"));
-            TRY(cuda_check(cudaStreamSynchronize(st), "state download"));
-        }
+        for (int f = 0; f < 4; f++) *field[f] = f == m ? ps->staging : nullptr;
+        patch_out_kernel<<<ew_blocks(nn), 256, 0, st>>>(p, nn);
+        TRY(cuda_check(cudaGetLastError(), "patch_out_kernel"));
+        TRY(cuda_check(cudaMemcpyAsync(dst[m], ps->staging, nn * 8, cudaMemcpyDeviceToHost, st),
+                       "state download"));
+        TRY(cuda_check(cudaStreamSynchronize(st), "state download"));
     }
     return SWA_OK;
 }
