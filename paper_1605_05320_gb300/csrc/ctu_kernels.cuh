@@ -28,46 +28,12 @@
 //      above)) and the update.
 // Each edge term is computed once per block instead of once per reading
 // cell.  Expressions and the order of every sum follow the FP64 reference, so
-// with contraction disabled (the FP64 instantiation) the rounding matches
-// it.
+// with contraction disabled the rounding matches it.  This is the FP64 step;
+// the FP32 one runs as warp strips (ctu_strips.cuh).
 #pragma once
 #include "fwd_kernels.cuh"
 
 namespace swadj {
-
-// Division and square root where the operand is a positive normal number
-// (depths, 2c, sums of square roots of depths): exact in FP64, the
-// reference's rounding; one-instruction approximations in FP32.
-__device__ __forceinline__ double ctu_div(double a, double b) { return a / b; }
-__device__ __forceinline__ float ctu_div(float a, float b) { return a * rcp_ftz(b); }
-__device__ __forceinline__ double ctu_sqrt(double x) { return sqrt(x); }
-__device__ __forceinline__ float ctu_sqrt(float x) { return x * rsqrt_ftz(x); }
-
-// The f-wave Roe solve of fwave_roe (FP64: that very function; FP32: the same
-// expressions with ctu_div / ctu_sqrt).
-template <typename R>
-__device__ __forceinline__ void ctu_roe(R g, R hL, R mnL, R mtL, R unL, R utL, R sqL, R etaL,
-                                        R hR, R mnR, R mtR, R unR, R utR, R sqR, R etaR,
-                                        R &uh, R &ch, R &b1, R &b2, R &b3, R &vh) {
-    if constexpr (sizeof(R) == 8) {
-        fwave_roe<R>(g, hL, mnL, mtL, unL, utL, sqL, etaL, hR, mnR, mtR, unR, utR, sqR, etaR,
-                     uh, ch, b1, b2, b3, vh);
-    } else {
-        const R hhat = R(0.5) * (hL + hR);
-        const R rden = rcp_ftz(sqL + sqR);
-        uh = (sqL * unL + sqR * unR) * rden;
-        vh = (sqL * utL + sqR * utR) * rden;
-        ch = ctu_sqrt(g * hhat);
-        const R s1 = uh - ch, s3 = uh + ch;
-        const R df1 = mnR - mnL;
-        const R df2 = (mnR * unR - mnL * unL) + g * hhat * (etaR - etaL);
-        const R df3 = mnR * utR - mnL * utL;
-        const R rw = rcp_ftz(s3 - s1);
-        b1 = (s3 * df1 - df2) * rw;
-        b3 = (df2 - s1 * df1) * rw;
-        b2 = df3 - vh * df1;
-    }
-}
 
 // Fluctuations of one edge (the first-order part of edge_flux, same sums).
 template <typename R>
@@ -98,9 +64,9 @@ __device__ __forceinline__ void ctu_tsplit(const Wave6<R> &w, const R a[3], R bm
     const R mu[3] = {vh - ch, vh, vh + ch};
     const R two_c = R(2) * ch;
     R beta[3];
-    beta[0] = ctu_div((vh + ch) * a[0] - a[2], two_c);
+    beta[0] = ((vh + ch) * a[0] - a[2]) / two_c;
     beta[1] = a[1] - uh * a[0];
-    beta[2] = ctu_div(a[2] - (vh - ch) * a[0], two_c);
+    beta[2] = (a[2] - (vh - ch) * a[0]) / two_c;
     const R r[3][3] = {{R(1), uh, vh - ch}, {R(0), R(1), R(0)}, {R(1), uh, vh + ch}};
 #pragma unroll
     for (int m = 0; m < 3; m++) { bm[m] = R(0); bp[m] = R(0); }
@@ -147,7 +113,7 @@ __device__ __forceinline__ void ctu_cell_terms(const Wave6<R> &lo, const Wave6<R
     M[0] = pm0[0] + pm1[0]; M[1] = pm0[2] + pm1[2]; M[2] = pm0[1] + pm1[1];
 }
 
-template <typename R, bool PERT, int TX, int TY>
+template <typename R, int TX, int TY>
 __global__ void __launch_bounds__(TX *TY)
 fwd_ctu_kernel(FwdParams<R> p) {
     using L = CtuSmem<R, TX, TY>;
@@ -209,22 +175,14 @@ fwd_ctu_kernel(FwdParams<R> p) {
         const R b = p.bath[o];
         if (fx) mu = -mu;
         if (fy) mv = -mv;
-        R h, eta;
-        if (PERT) { eta = a; h = a + b; }
-        else { h = a; eta = a + b; }
+        const R h = a, eta = a + b;
         s_h[r] = h;
         s_mu[r] = mu;
         s_mv[r] = mv;
         s_eta[r] = eta;
-        if constexpr (sizeof(R) == 8) {
-            s_u[r] = mu / h;
-            s_v[r] = mv / h;
-        } else {
-            const R rh = rcp_ftz(h);
-            s_u[r] = mu * rh;
-            s_v[r] = mv * rh;
-        }
-        s_sq[r] = ctu_sqrt(h);
+        s_u[r] = mu / h;
+        s_v[r] = mv / h;
+        s_sq[r] = sqrt(h);
     }
     __syncthreads();
 
@@ -232,14 +190,14 @@ fwd_ctu_kernel(FwdParams<R> p) {
     //    edge frames (h, hu, hv) / (h, hv, hu); the cell's own state is kept
     //    in registers (phase C overwrites the staging area)
     const int cx = tx + H, cy = ty + H, cc = cy * RX + cx;
-    const R a0 = PERT ? s_eta[cc] : s_h[cc], mu0 = s_mu[cc], mv0 = s_mv[cc];
+    const R a0 = s_h[cc], mu0 = s_mu[cc], mv0 = s_mv[cc];
     constexpr int NBX = (RY - 2) * (RX - 1), NBY = (RY - 1) * (RX - 2);
     for (int e = tid; e < NBX + NBY; e += NT) {
         Wave6<R> w;
         if (e < NBX) {
             const int ry = 1 + e / (RX - 1), k = e % (RX - 1);
             const int a = ry * RX + k, b = a + 1;
-            ctu_roe<R>(p.g, s_h[a], s_mu[a], s_mv[a], s_u[a], s_v[a], s_sq[a], s_eta[a],
+            fwave_roe<R>(p.g, s_h[a], s_mu[a], s_mv[a], s_u[a], s_v[a], s_sq[a], s_eta[a],
                        s_h[b], s_mu[b], s_mv[b], s_u[b], s_v[b], s_sq[b], s_eta[b], w.uh,
                        w.ch, w.b1, w.b2, w.b3, w.vh);
             wave_put(wxa, NWX, ry * (RX - 1) + k, w);
@@ -247,7 +205,7 @@ fwd_ctu_kernel(FwdParams<R> p) {
             const int f = e - NBX;
             const int k = f / (RX - 2), rx = 1 + f % (RX - 2);
             const int a = k * RX + rx, b = a + RX;
-            ctu_roe<R>(p.g, s_h[a], s_mv[a], s_mu[a], s_v[a], s_u[a], s_sq[a], s_eta[a],
+            fwave_roe<R>(p.g, s_h[a], s_mv[a], s_mu[a], s_v[a], s_u[a], s_sq[a], s_eta[a],
                        s_h[b], s_mv[b], s_mu[b], s_v[b], s_u[b], s_sq[b], s_eta[b], w.uh,
                        w.ch, w.b1, w.b2, w.b3, w.vh);
             wave_put(wya, NWY, k * RX + rx, w);
@@ -320,21 +278,16 @@ fwd_ctu_kernel(FwdParams<R> p) {
     double s_cell = 0.0;
     if (gi < nx && gj < ny) {
         const size_t o = (size_t)gj * nx + gi;
-        const R hn = PERT ? n0 + p.bath[o] : n0;
+        const R hn = n0;
         o0[o] = n0;
         o1[o] = n1;
         o2[o] = n2;
         if (!(hn > R(0)) || !isfinite(n1) || !isfinite(n2)) atomicOr(p.err, ERR_UNSTABLE);
-        if (PERT) {
-            s_cell = (double)cfl_f32((float)hn, (float)n1, (float)n2, (float)p.g,
-                                     1.f / (float)p.dx, 1.f / (float)p.dy, 1);
-        } else {
-            const R c = sqrt(p.g * hn);
-            R s = (fabs(n1 / hn) + c) / p.dx;
-            const R sy = (fabs(n2 / hn) + c) / p.dy;
-            if (sy > s) s = sy;
-            s_cell = (double)s;
-        }
+        const R c = sqrt(p.g * hn);
+        R s = (fabs(n1 / hn) + c) / p.dx;
+        const R sy = (fabs(n2 / hn) + c) / p.dy;
+        if (sy > s) s = sy;
+        s_cell = (double)s;
         if (!(s_cell >= 0.0)) s_cell = 0.0;
     }
 
@@ -368,20 +321,20 @@ fwd_ctu_kernel(FwdParams<R> p) {
     }
 }
 
-template <typename R, bool PERT, int TX, int TY>
+template <typename R, int TX, int TY>
 int ctu_launch(FwdParams<R> p, cudaStream_t st, const char *name) {
     constexpr size_t smem = CtuSmem<R, TX, TY>::bytes;
     static_assert(smem <= 227 * 1024, "tile does not fit in shared memory");
     // set on every launch: the attribute belongs to the current device
     const int rc = swadj_host::cuda_check(
-        cudaFuncSetAttribute(fwd_ctu_kernel<R, PERT, TX, TY>,
+        cudaFuncSetAttribute(fwd_ctu_kernel<R, TX, TY>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
         name);
     if (rc) return rc;
     dim3 grid((p.nx + TX - 1) / TX, (p.ny + TY - 1) / TY);
     p.nblocks = (int)(grid.x * grid.y);
     return swadj_host::cuda_check(
-        launch_chained(fwd_ctu_kernel<R, PERT, TX, TY>, grid, dim3(TX, TY), smem, st, p), name);
+        launch_chained(fwd_ctu_kernel<R, TX, TY>, grid, dim3(TX, TY), smem, st, p), name);
 }
 
 template <int TX, int TY>

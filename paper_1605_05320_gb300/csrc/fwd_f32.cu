@@ -11,7 +11,7 @@
 // arithmetic.  The CFL maximum
 // is reduced in float (max is exact); the last block to finish turns it into
 // the next time step in double.
-#include "ctu_kernels.cuh"
+#include "ctu_strips.cuh"
 #include "strips.cuh"
 
 namespace swadj {
@@ -24,8 +24,10 @@ namespace f32 {
 // Where the ocean is at rest a unit costs little (strips.cuh), so units are
 // short and taken as warps free up: the active part of the domain spreads
 // over every SM instead of over the few warps whose strips it crosses.
-// ORD: the order of the scheme (1 or 2), fixed at compile time.
-template <int ORD>
+// ORD: the order of the scheme (1 or 2), fixed at compile time; CTU: the
+// unsplit update with transverse waves (a window at rest stays so under it
+// too, with the same CFL terms).
+template <int ORD, bool CTU>
 __global__ void __launch_bounds__(strip::kThreads, 4)
     fwd_f32_strips(FwdParams<float> p, int rows, int nunits) {
     __shared__ float s_nu[2];
@@ -75,8 +77,12 @@ __global__ void __launch_bounds__(strip::kThreads, 4)
         }
         // Units with waves take the full path: quiet units cover the ocean
         // at rest, and the strip loop without its row skipping is leaner.
-        strip::strip_unit<ORD, 2>(v, sx * strip::kOut, sy * rows, rows, s_nu[0], s_nu[1], p.g,
-                               ring[threadIdx.x >> 5], smax, bad);
+        if (CTU)
+            strip::ctu_unit<ORD>(v, sx * strip::kOut, sy * rows, rows, s_nu[0], s_nu[1], p.g,
+                                 ring[threadIdx.x >> 5], smax, bad);
+        else
+            strip::strip_unit<ORD, 2>(v, sx * strip::kOut, sy * rows, rows, s_nu[0], s_nu[1], p.g,
+                                      ring[threadIdx.x >> 5], smax, bad);
     }
     if (bad) atomicOr(p.err, ERR_UNSTABLE);
     fwave::finish_step<strip::kThreads>(p.clk, p.partial, p.nblocks, p.cfl, smax, red, &am_last,
@@ -184,13 +190,14 @@ constexpr int kMaxStepBlocks = 4096;
 
 
 // Blocks of one resident wave of the strip kernel on the current device.
+template <bool CTU>
 static int resident_blocks() {
     static int blocks = 0;
     if (blocks == 0) {
         int dev = 0, sms = 0, per_sm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f32::fwd_f32_strips<2>,
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f32::fwd_f32_strips<2, CTU>,
                                                       strip::kThreads, 0);
         blocks = (sms > 0 ? sms : 1) * (per_sm > 0 ? per_sm : 1);
         if (blocks > kMaxStepBlocks) blocks = kMaxStepBlocks;
@@ -216,9 +223,10 @@ static int strip_units(int nx, int ny, int rows) {
 // 30.1 / 23.9 and 32.8 / 28.7; 1500^2 (34 rows) 33.9 / 35.4 and 53.3 / 44.4;
 // 2048^2 keeps 32; 4096^2 (36 rows) 84.3 / 86.1 and 258 / 248.
 constexpr int kMaxUnitRows = 36;
+template <bool CTU>
 static int unit_rows(const FwdParams<float> &p) {
     if (p.fwd_rows > 0) return p.fwd_rows;
-    const long long warps = (long long)resident_blocks() * (strip::kThreads / 32);
+    const long long warps = (long long)resident_blocks<CTU>() * (strip::kThreads / 32);
     const int nsx = (p.nx + strip::kOut - 1) / strip::kOut;
     long long k = ((long long)nsx + warps - 1) / warps;
     for (;; k++) {
@@ -228,22 +236,23 @@ static int unit_rows(const FwdParams<float> &p) {
     }
 }
 
+template <bool CTU>
+static int launch_strips(FwdParams<float> p, cudaStream_t st) {
+    const int rows = unit_rows<CTU>(p);
+    const int units = strip_units(p.nx, p.ny, rows);
+    constexpr int wpb = strip::kThreads / 32;
+    const int blocks = (units + wpb - 1) / wpb, wave = resident_blocks<CTU>();
+    p.nblocks = blocks < wave ? blocks : wave;
+    return swadj_host::cuda_check(
+        launch_chained(p.order == 2 ? f32::fwd_f32_strips<2, CTU> : f32::fwd_f32_strips<1, CTU>,
+                       p.nblocks, strip::kThreads, 0, st, p, rows, units),
+        "fwd_f32_strips");
+}
+
 template <>
 int fwd_launch_step<float>(const FwdParams<float> &p0, cudaStream_t st) {
+    if (p0.two_d) return launch_strips<false>(p0, st);
     FwdParams<float> p = p0;
-    if (p.two_d) {
-        const int rows = unit_rows(p);
-        const int units = strip_units(p.nx, p.ny, rows);
-        constexpr int wpb = strip::kThreads / 32;
-        int blocks = (units + wpb - 1) / wpb;
-        const int wave = resident_blocks();
-        if (blocks > wave) blocks = wave;
-        p.nblocks = blocks;
-        return swadj_host::cuda_check(
-            launch_chained(p.order == 2 ? f32::fwd_f32_strips<2> : f32::fwd_f32_strips<1>,
-                           p.nblocks, strip::kThreads, 0, st, p, rows, units),
-            "fwd_f32_strips");
-    }
     dim3 grid((p.nx + 255) / 256, 1);
     p.nblocks = (int)grid.x;
     return swadj_host::cuda_check(launch_chained(f32::fwd_f32_1d, grid, 256, 0, st, p),
@@ -291,12 +300,12 @@ int fwd_wd_blocks<float>(const FwdParams<float> &p) {
 
 template <>
 int fwd_launch_ctu<float>(const FwdParams<float> &p, cudaStream_t st) {
-    return ctu_launch<float, true, 32, 16>(p, st, "fwd_ctu_kernel<float>");
+    return launch_strips<true>(p, st);
 }
 
 template <>
 int fwd_ctu_blocks<float>(const FwdParams<float> &p) {
-    return ctu_blocks<32, 16>(p.nx, p.ny);
+    return fwd_step_blocks<float>(p);
 }
 
 template <>

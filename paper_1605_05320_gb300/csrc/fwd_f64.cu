@@ -92,7 +92,7 @@ int fwd_wd_blocks<double>(const FwdParams<double> &p) {
 
 template <>
 int fwd_launch_ctu<double>(const FwdParams<double> &p, cudaStream_t st) {
-    return ctu_launch<double, false, 16, 8>(p, st, "fwd_ctu_kernel<double>");
+    return ctu_launch<double, 16, 8>(p, st, "fwd_ctu_kernel<double>");
 }
 
 template <>

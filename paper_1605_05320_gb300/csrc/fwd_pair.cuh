@@ -73,9 +73,9 @@ struct Cell {
 
 // Waves of one edge: speeds s1 = uh - ch, s3 = uh + ch (and uh of the shear
 // wave), the tangential Roe velocity and the strengths of the waves
-// b1 (1, s1, vh), b2 (0, 0, 1), b3 (1, s3, vh).
+// b1 (1, s1, vh), b2 (0, 0, 1), b3 (1, s3, vh); hr = 1 / (2 ch).
 struct Edge {
-    float s1, s3, vh, b1, b2, b3, uh;
+    float s1, s3, vh, b1, b2, b3, uh, ch, hr;
 };
 
 // The upwind neighbour of wave 1 or 3 for the limiter: its speed, tangential
@@ -107,7 +107,10 @@ __device__ __forceinline__ Cell derive(float eta, float h, float mn, float mt) {
 // vhat sqrt(h)-weighted ((sqrt(hL) uL + sqrt(hR) uR) / (sqrt(hL) +
 // sqrt(hR))), chat = sqrt(g hhat); the momentum jump carries the bathymetry
 // source as g hhat (etaR - etaL), so the ocean at rest has no waves.
-// 1 / (s3 - s1) = 1 / (2 chat) comes from the same rsqrt as chat.
+// 1 / (s3 - s1) = 1 / (2 chat) comes from the same rsqrt as chat, or, RCP (the
+// unsplit step), from a reciprocal of s3 - s1, with which the waves' momenta
+// add up to the jump to one rounding.
+template <bool RCP = false>
 __device__ __forceinline__ Edge solve(float g_half, const Cell &L, const Cell &R) {
     Edge w;
     const float gh = mul(g_half, add(L.h, R.h));   // g hhat
@@ -116,50 +119,61 @@ __device__ __forceinline__ Edge solve(float g_half, const Cell &L, const Cell &R
     w.uh = uv.x;
     w.vh = uv.y;
     const float rc = rsq(gh);
-    const float ch = mul(gh, rc);
-    w.s1 = sub(w.uh, ch);
-    w.s3 = add(w.uh, ch);
+    w.ch = mul(gh, rc);
+    w.s1 = sub(w.uh, w.ch);
+    w.s3 = add(w.uh, w.ch);
     const float df1 = sub(R.mn, L.mn);
     const f2 dPT = fma(mk(L.P, L.T), dup(-1.f), mk(R.P, R.T));
     const float df2 = fma(gh, sub(R.eta, L.eta), dPT.x);
-    const float hr = mul(0.5f, rc);
-    const f2 b = mul(mk(fms(w.s3, df1, df2), fnma(w.s1, df1, df2)), dup(hr));
+    w.hr = RCP ? rcp(sub(w.s3, w.s1)) : mul(0.5f, rc);
+    const f2 b = mul(mk(fms(w.s3, df1, df2), fnma(w.s1, df1, df2)), dup(w.hr));
     w.b1 = b.x;
     w.b3 = b.y;
     w.b2 = fnma(w.vh, df1, dPT.y);
     return w;
 }
 
+// Fluctuations of an edge as pairs (A-dQ, A+dQ), one per component.  A wave
+// of speed s goes right with weight (1 + sign s)/2 (half each way at s = 0).
+// SUB: the edge is subsonic (s1 < 0 < s3), so wave 1 goes left and wave 3
+// right.
+struct Fluct {
+    f2 a0, a1, a2;
+};
+template <bool SUB>
+__device__ __forceinline__ Fluct fluct(const Edge &w) {
+    Fluct f;
+    if (SUB) {
+        f.a0 = mk(w.b1, w.b3);
+        f.a1 = mul(f.a0, mk(w.s1, w.s3));
+    } else {
+        const float p1 = mul(fma(0.5f, sgn(w.s1), 0.5f), w.b1);
+        const float p3 = mul(fma(0.5f, sgn(w.s3), 0.5f), w.b3);
+        const float e1 = sub(w.b1, p1), e3 = sub(w.b3, p3);
+        f.a0 = mk(add(e1, e3), add(p1, p3));
+        f.a1 = mk(fma(e1, w.s1, mul(e3, w.s3)), fma(p1, w.s1, mul(p3, w.s3)));
+    }
+    const float p2 = mul(fma(0.5f, sgn(w.uh), 0.5f), w.b2);
+    f.a2 = fma(f.a0, dup(w.vh), mk(sub(w.b2, p2), p2));
+    return f;
+}
+
 // Fluctuations and MC-limited correction of edge w: L = A-dQ + F into the
-// left cell, R = A+dQ - F into the right cell.  A wave of speed s goes right
-// with weight (1 + sign s)/2 (half each way at s = 0); F = sum_p sign(s^p)/2
-// (1 - nu |s^p|) phi(theta^p) Z^p, computed as (sign(s) - nu s) times half
-// the limited strength (the same number).  u1, u3: the upwind neighbours of
-// waves 1 and 3 (the left edge for s > 0, the right one otherwise); b2l,
-// b2r: the shear-wave strengths of the left and right edges.  SUB: every
-// edge of w is subsonic (s1 < 0 < s3), so wave 1 goes left and wave 3 right.
+// left cell, R = A+dQ - F into the right cell.  F = sum_p sign(s^p)/2 (1 - nu
+// |s^p|) phi(theta^p) Z^p, computed as (sign(s) - nu s) times half the limited
+// strength (the same number).  u1, u3: the upwind neighbours of waves 1 and
+// 3 (the left edge for s > 0, the right one otherwise); b2l, b2r: the
+// shear-wave strengths of the left and right edges.
 template <bool SUB>
 __device__ __forceinline__ Net net(const Edge &w, const Up &u1, const Up &u3, float b2l,
-                                   float b2r, float nu, int order) {
-    const float g2 = sgn(w.uh);
-    const f2 s = mk(w.s1, w.s3), b = mk(w.b1, w.b3);
-    f2 a0, a1, k;   // (A-dQ, A+dQ) components 0 and 1; (sign(s) - nu s) of (-wave 1, wave 3)
-    if (SUB) {
-        a0 = b;
-        a1 = mul(b, s);
-        k = fma(mk(nu, -nu), s, dup(1.f));
-    } else {
-        const float g1 = sgn(w.s1), g3 = sgn(w.s3);
-        const float p1 = mul(fma(0.5f, g1, 0.5f), w.b1), p3 = mul(fma(0.5f, g3, 0.5f), w.b3);
-        const float e1 = sub(w.b1, p1), e3 = sub(w.b3, p3);
-        a0 = mk(add(e1, e3), add(p1, p3));
-        a1 = mk(fma(e1, w.s1, mul(e3, w.s3)), fma(p1, w.s1, mul(p3, w.s3)));
-        k = mk(-fnma(nu, w.s1, g1), fnma(nu, w.s3, g3));
-    }
-    const float p2 = mul(fma(0.5f, g2, 0.5f), w.b2), e2 = sub(w.b2, p2);
-    const f2 a2 = fma(a0, dup(w.vh), mk(e2, p2));
+                                   float b2r, float nu, int order, const Fluct &f) {
+    f2 a0 = f.a0, a1 = f.a1, a2 = f.a2;
     Net n;
     if (order >= 2) {
+        const float g2 = sgn(w.uh);
+        const f2 s = mk(w.s1, w.s3), b = mk(w.b1, w.b3);
+        const f2 k = SUB ? fma(mk(nu, -nu), s, dup(1.f))   // sign(s) - nu s of (-wave 1, wave 3)
+                         : mk(-fnma(nu, w.s1, sgn(w.s1)), fnma(nu, w.s3, sgn(w.s3)));
         // theta^p b^p = b_up (1 + s_up s + v_up vhat) / (1 + s^2 + vhat^2)
         const f2 m = fma(s, s, dup(fma(w.vh, w.vh, 1.f)));
         const f2 d = fma(mk(u1.s, u3.s), s, fma(mk(u1.vh, u3.vh), dup(w.vh), dup(1.f)));
@@ -172,13 +186,10 @@ __device__ __forceinline__ Net net(const Edge &w, const Up &u1, const Up &u3, fl
         const f2 lr = mk(1.f, -1.f);
         a0 = fma(dup(F0), lr, a0);
         a1 = fma(dup(F1), lr, a1);
-        const f2 q2 = fma(dup(F2), lr, a2);
-        n.L2 = q2.x; n.R2 = q2.y;
-    } else {
-        n.L2 = a2.x; n.R2 = a2.y;
+        a2 = fma(dup(F2), lr, a2);
     }
-    n.L0 = a0.x; n.L1 = a1.x;
-    n.R0 = a0.y; n.R1 = a1.y;
+    n.L0 = a0.x; n.L1 = a1.x; n.L2 = a2.x;
+    n.R0 = a0.y; n.R1 = a1.y; n.R2 = a2.y;
     return n;
 }
 
@@ -199,10 +210,10 @@ __device__ __forceinline__ Net net3(const Edge &wl, const Edge &w, const Edge &w
     if (all_sub) {
         u1.s = wr.s1; u1.vh = wr.vh; u1.b = wr.b1;
         u3.s = wl.s3; u3.vh = wl.vh; u3.b = wl.b3;
-        return net<true>(w, u1, u3, wl.b2, wr.b2, nu, order);
+        return net<true>(w, u1, u3, wl.b2, wr.b2, nu, order, fluct<true>(w));
     }
     upwind(w, wl, wr, u1, u3);
-    return net<false>(w, u1, u3, wl.b2, wr.b2, nu, order);
+    return net<false>(w, u1, u3, wl.b2, wr.b2, nu, order, fluct<false>(w));
 }
 
 }  // namespace fp

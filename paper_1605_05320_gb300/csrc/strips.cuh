@@ -56,8 +56,7 @@ struct Nb1 {
 // values (wave 1 from the right edge, wave 3 from the left, both shear
 // strengths), otherwise both neighbours in full.
 template <class NB, bool SUB, int ORD>
-__device__ __forceinline__ fp::Net xnet(const fp::Edge &w,
-                                                        float nu) {
+__device__ __forceinline__ fp::Net xnet(const fp::Edge &w, float nu, const fp::Fluct &f) {
     fp::Up u1 = {}, u3 = {};
     if (SUB) {
         float b2l = w.b2, b2r = w.b2;
@@ -66,7 +65,7 @@ __device__ __forceinline__ fp::Net xnet(const fp::Edge &w,
             u3.s = NB::l(w.s3); u3.vh = NB::l(w.vh); u3.b = NB::l(w.b3);
             b2l = NB::l(w.b2); b2r = NB::r(w.b2);
         }
-        return fp::net<true>(w, u1, u3, b2l, b2r, nu, ORD);
+        return fp::net<true>(w, u1, u3, b2l, b2r, nu, ORD, f);
     }
     fp::Edge wl = w, wr = w;
     if (ORD >= 2) {
@@ -76,19 +75,19 @@ __device__ __forceinline__ fp::Net xnet(const fp::Edge &w,
         wr.b1 = NB::r(w.b1); wr.b2 = NB::r(w.b2); wr.b3 = NB::r(w.b3);
     }
     fp::upwind(w, wl, wr, u1, u3);
-    return fp::net<false>(w, u1, u3, wl.b2, wr.b2, nu, ORD);
+    return fp::net<false>(w, u1, u3, wl.b2, wr.b2, nu, ORD, f);
 }
 
 // The x-edge(s) a lane solves, between its cell and its right neighbour
 // (x frame: mn = hu, mt = hv).
-template <class NB>
+template <class NB, bool RCP = false>
 __device__ __forceinline__ fp::Edge xsolve(const fp::Cell &c,
                                                            float g_half) {
     fp::Cell r;
     r.h = NB::r(c.h); r.mn = NB::r(c.mn); r.mt = c.mt; r.sq = NB::r(c.sq);
     r.su = NB::r(c.su); r.sv = NB::r(c.sv); r.P = NB::r(c.P); r.T = NB::r(c.T);
     r.eta = NB::r(c.eta);
-    return fp::solve(g_half, c, r);
+    return fp::solve<RCP>(g_half, c, r);
 }
 
 // The x-swept cell(s) in the y frame (mn = hv) from a lane's cell c and its
@@ -98,7 +97,7 @@ template <class NB, bool SUB, int ORD>
 __device__ __forceinline__ fp::Cell xsweep(const fp::Cell &c,
                                                            const fp::Edge &w,
                                                            float nux) {
-    const fp::Net n = xnet<NB, SUB, ORD>(w, nux);
+    const fp::Net n = xnet<NB, SUB, ORD>(w, nux, fp::fluct<SUB>(w));
     const float mnu = -nux;
     const float d0 = fp::mul(mnu, fp::add(NB::l(n.R0), n.L0));
     const float d1 = fp::mul(mnu, fp::add(NB::l(n.R1), n.L1));
