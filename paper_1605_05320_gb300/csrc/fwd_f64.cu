@@ -66,11 +66,20 @@ static int launch_sweeps(const FwdParams<double> &p, cudaStream_t st) {
     return rc ? rc : launch_sweep<true, WD>(p, sms, st);
 }
 
+template <bool WD>
+static int launch_line(const FwdParams<double> &p, cudaStream_t st) {
+    // at most kInitBlocks blocks (the reduction slots every grid has)
+    const int units = (p.nx + s64::kLineOut - 1) / s64::kLineOut;
+    const int blocks = units < kInitBlocks ? units : kInitBlocks;
+    auto kernel = p.order == 2 ? s64::fwd_f64_line<WD, 2> : s64::fwd_f64_line<WD, 1>;
+    return swadj_host::cuda_check(launch_chained(kernel, blocks, 32, 0, st, p), "fwd_f64_line");
+}
+
 template <>
 int fwd_launch_step<double>(const FwdParams<double> &p, cudaStream_t st) {
     if (p.two_d && p.keep_input) return launch_step<double, false, true, 32, 4>(p, st);
     if (p.two_d) return launch_sweeps<false>(p, st);
-    return launch_step<double, false, false, 128, 1>(p, st);
+    return launch_line<false>(p, st);
 }
 
 template <>
@@ -82,7 +91,7 @@ int fwd_step_blocks<double>(const FwdParams<double> &p) {
 template <>
 int fwd_launch_wd<double>(const FwdParams<double> &p, cudaStream_t st) {
     if (p.two_d) return launch_sweeps<true>(p, st);
-    return launch_step<double, false, false, 128, 1, true>(p, st);
+    return launch_line<true>(p, st);
 }
 
 template <>

@@ -367,5 +367,121 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
 }
 
+// ------------------------------------------------------------- 1D grids
+// One step of a 1D grid: a warp per 28 output cells (32 with two halo cells
+// each side), a cell and the edge to its right per lane, neighbours by
+// shuffles.  A 1D grid has few cells, so what counts is how long one warp
+// takes: about 115 FP64 operations a lane (the tiled kernel: about 360, each
+// edge limited twice), with warps spread over as many schedulers as there
+// are.
+// Measured, us per step, tiles / strips: 100 cells 28.8 / 10.7, 2000 31.1 / 12.7
+// (14.5 not chained), 8000 31.3 / 12.9; 2000 with wet/dry 50 / 20.6.
+__device__ __forceinline__ double dn(double x) { return __shfl_down_sync(0xffffffffu, x, 1); }
+__device__ __forceinline__ double up(double x) { return __shfl_up_sync(0xffffffffu, x, 1); }
+
+constexpr int kLineOut = 28;
+template <bool WD, int ORD>
+__global__ void __launch_bounds__(32) fwd_f64_line(FwdParams<double> p) {
+    chain_begin();
+    volatile DevClock *clk = p.clk;
+    const double t = clk->t;
+    double dt = clk->dt_cfl;
+    if (p.t_end - t < dt) dt = p.t_end - t;
+    if (!(dt > 0.0)) return;   // clock already at t_end: no-op step
+    const int cur = clk->cur, lane = threadIdx.x;
+    const double *q0 = p.q[cur][0], *q1 = p.q[cur][1];
+    const double g = p.g, tol = p.dry_tol, nu = dt / p.dx;
+    double mx = 0.0;   // max |u| + c
+    bool bad = false;
+    const int units = (p.nx + kLineOut - 1) / kLineOut;
+    const int ngroups = p.gauges.n > 0 ? (p.gauges.n + 31) / 32 : 0;
+    for (int unit = blockIdx.x; unit < units + ngroups; unit += gridDim.x) {
+        if (unit >= units) {
+            record_gauge_group<double>(p.gauges, q0, p.bath, p.nx, p.ny, 0, p.clk, unit - units);
+            continue;
+        }
+        const int i = unit * kLineOut - 2 + lane;
+        bool flip;
+        const int o = ghost_index(i, p.nx, p.bc.lo_x, p.bc.hi_x, &flip);
+        const double h = q0[o], b = p.bath[o];
+        const double m = flip ? -q1[o] : q1[o];
+        const Cell c = derive<WD>(tol, h, m, 0.0, h + b, b, true);
+        Cell r;
+        r.h = dn(c.h); r.mn = dn(c.mn); r.mt = 0.0; r.eta = dn(c.eta); r.un = dn(c.un);
+        r.ut = 0.0; r.sq = dn(c.sq); r.b = dn(c.b);
+        const bool still = __all_sync(0xffffffffu, is_still<WD>(tol, c, r));
+        Edge w = {};
+        if (!still) w = solve<WD>(g, tol, c, r);   // edge (i|i+1)
+        double F[3] = {0.0, 0.0, 0.0};
+        if (ORD >= 2) {
+            Edge wl = {}, wr = {};
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                wl.z1[k] = up(w.z1[k]); wl.z3[k] = up(w.z3[k]);
+                wr.z1[k] = dn(w.z1[k]); wr.z3[k] = dn(w.z3[k]);
+            }
+            if (!still && (!WD || !w.shore)) correct(wl, w, wr, nu, F);
+        }
+        double q[2] = {c.h, c.mn};
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+            const double apl = up(w.ap[k]), Fl = up(F[k]);
+            if (!still) {
+                double d = -nu * (apl + w.am[k]);
+                if (ORD >= 2) d = d - nu * (F[k] - Fl);
+                q[k] = q[k] + d;
+            }
+        }
+        const bool dry = WD && !(q[0] > tol);
+        if (dry) {   // a dry cell keeps no momentum, no negative depth
+            if (q[0] < 0.0) q[0] = 0.0;
+            q[1] = 0.0;
+        }
+        if (lane >= 2 && lane < 30 && i < p.nx) {
+            p.q[cur ^ 1][0][i] = q[0];
+            p.q[cur ^ 1][1][i] = q[1];
+            bad |= !(WD ? q[0] >= 0.0 : q[0] > 0.0) || !isfinite(q[1]);
+            if (!dry) {
+                const double ax = fabs(div(q[1], recip(q[0]))) + root(g * q[0]);
+                if (!is_nan(ax)) mx = max_pos(mx, ax);
+            }
+        }
+    }
+    if (bad) atomicOr(p.err, ERR_UNSTABLE);
+    mx = mx / p.dx;
+    for (int s = 16; s > 0; s >>= 1) {
+        const double v = __shfl_xor_sync(0xffffffffu, mx, s);
+        mx = v > mx ? v : mx;
+    }
+    int last = 0;
+    if (lane == 0) {
+        p.partial[blockIdx.x] = mx;
+        __threadfence();
+        last = atomicAdd((unsigned int *)&p.clk->ticket, 1u) == gridDim.x - 1;
+    }
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
+    __threadfence();
+    mx = 0.0;
+    for (int k = lane; k < (int)gridDim.x; k += 32) {
+        const double v = __ldcg(p.partial + k);
+        mx = v > mx ? v : mx;
+    }
+    for (int s = 16; s > 0; s >>= 1) {
+        const double v = __shfl_xor_sync(0xffffffffu, mx, s);
+        mx = v > mx ? v : mx;
+    }
+    if (lane == 0) {
+        clk->t = t + dt;
+        clk->smax = mx;
+        clk->dt_cfl = p.cfl / mx;
+        clk->cur = cur ^ 1;
+        clk->nsteps = clk->nsteps + 1;
+        clk->ticket = 0u;
+        clk->work = 0u;
+        clk->work2 = 0u;
+        if (p.gauges.n > 0) *p.gauges.row += 1;
+    }
+}
+
 }  // namespace s64
 }  // namespace swadj
