@@ -26,8 +26,7 @@ struct AdjParams {
     int two_steps;
     // FP32 2D one-step kernel: no cell is dry (no wall edges to check)
     int all_wet;
-    // FP32 2D one-step kernel: 1 = the unit has had a nonzero value at an
-    // earlier step (it skips the quiet scan); null: no quiet scan
+    // FP32 2D one-step kernel: marks of its units; null: no quiet scan
     unsigned char *umap;
     int umap_n;
 };

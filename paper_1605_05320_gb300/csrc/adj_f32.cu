@@ -205,16 +205,28 @@ __global__ void __launch_bounds__(256, 4) adj_f32_strips(AdjParams<float> p, int
     // upper boundary need no mapping; past the last row the load is clamped
     // and its values unused)
     const bool yin = y0 - 2 >= 0 && ylast + 2 < p.ny;
-    // A unit that has had a nonzero value keeps having them: it skips the
-    // quiet scan (the map is only a hint; the scan alone decides quiet).
-    const bool scan = p.umap && (unit >= p.umap_n || p.umap[unit] == 0);
-    if (scan && quiet_a(p, col, y0, ylast, yin)) {   // quiet: the unit stays zero
+    // A unit zero in both buffers among units that are stays so and needs no
+    // scan and no stores but a snapshot's (up to the sign of a zero).  A unit
+    // that has had a nonzero value keeps having them: it skips the scan.
+    // The zero part of a large grid was bound by the scan's loads and the
+    // zeros' stores; us per step, each unit scanned and stored / this, early
+    // and late in the zero phase: 2048^2 17.5 / 10.5 and 34.2 / 29.5, 4096^2
+    // 68 / 13 and 76 / 36.  Where most units are active the nine marks cost
+    // what they save: 512^2 5.9 / 6.1, 1024^2 8.0 / 6.9 and 12.8 / 13.0.
+    int own = UNIT_ACTIVE;
+    const bool still = p.umap && still_around(p.umap, sx, sy, nsx, nsy, own);
+    if (still && !p.snap_f && !p.snap_d) return;
+    const bool scan = own != UNIT_ACTIVE;
+    if (still || (scan && quiet_a(p, col, y0, ylast, yin))) {   // quiet: the unit stays zero
+        if (lane == 0) p.umap[unit] = UNIT_STILL;
         if (out) {
             for (int j = y0; j <= ylast; j++) {
                 const size_t o = (size_t)j * p.nx + gi;
-                p.dst[0][o] = 0.f;
-                p.dst[1][o] = 0.f;
-                p.dst[2][o] = 0.f;
+                if (!still) {
+                    p.dst[0][o] = 0.f;
+                    p.dst[1][o] = 0.f;
+                    p.dst[2][o] = 0.f;
+                }
                 if (p.snap_f) {
                     __stcs(p.snap_f + o, 0.f);
                     __stcs(p.snap_f + p.snap_comp_stride + o, 0.f);
@@ -228,7 +240,7 @@ __global__ void __launch_bounds__(256, 4) adj_f32_strips(AdjParams<float> p, int
         }
         return;
     }
-    if (scan && lane == 0 && unit < p.umap_n) p.umap[unit] = 1;
+    if (scan && lane == 0) p.umap[unit] = UNIT_ACTIVE;
     // Rows stream through the warp's ring of shared memory by cp.async,
     // kRingA - 1 rows ahead of the one read, in the order they are used:
     // y0 - 2, y0 - 1, ..., ylast + 3 (past the last row the fetch is
@@ -429,6 +441,10 @@ __device__ __forceinline__ CellA ghost_row(int r, int ny, int bc_lo, int bc_hi, 
 
 __global__ void __launch_bounds__(256, 3) adj_f32_strips2(AdjParams<float> p) {
     chain_begin();
+    // the marks of the one-step kernel's units do not hold after this step
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; p.umap && k < p.umap_n;
+         k += gridDim.x * blockDim.x)
+        p.umap[k] = UNIT_UNKNOWN;
     const int lane = threadIdx.x & 31;
     const int nsx = (p.nx + kOut2 - 1) / kOut2, nsy = (p.ny + kRows2 - 1) / kRows2;
     const int unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -516,10 +532,9 @@ int adj_f32_unit_map_bytes(int nx, int ny) {
 // walks its rows one after the other) and takes the lowest strips that still
 // fill the warps; on larger grids low strips follow the front of the still
 // zero adjoint more closely, at the price of four halo rows each.
-// Measured, us per step late in the solve, 32 rows / this rule: 64^2 18.5 /
-// 6.3, 512^2 18.5 / 8.2, 1024^2 18.5 / 14.4; 2048^2 (16 rows) 38.9 / 36.4 and
-// 25.9 / 24.9 early (8 rows: 38.5 and 24.1, 64: 43.4 and 33.5); 4096^2 (18)
-// 82.8 / 80.5.
+// Measured when the rule was made, us per step late in the solve, 32 rows /
+// this rule: 64^2 18.5 / 6.3, 512^2 18.5 / 8.2, 1024^2 18.5 / 14.4; 2048^2
+// (16 rows) 38.9 / 36.4 (8 rows: 38.5, 64: 43.4); 4096^2 (18) 82.8 / 80.5.
 static int adj_rows(int nx, int ny) {
     static long long warps = 0;
     if (warps == 0) {

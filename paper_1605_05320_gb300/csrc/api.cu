@@ -586,7 +586,7 @@ struct swa_adjoint {
     int steps_per_pass;   // FP32 2D: 1 or 2 adjoint steps per launch
     int all_wet;          // no cell with hbar <= dry_tol (no wall edges)
     double t_f;
-    unsigned char *umap;  // FP32 2D: units that have had a nonzero value (quiet-unit hint)
+    unsigned char *umap;  // FP32 2D: marks of the step's units
     int umap_n;
 };
 
@@ -909,7 +909,7 @@ int swa_set_adjoint_state(swa_adjoint *a, const double *phi, int where, void *st
             TRY(adj_in(a, k, 1, a->staging, st));
         }
     }
-    if (a->umap)   // a new state: no unit has had a nonzero value yet
+    if (a->umap)   // a new state: nothing is known of the step's units
         TRY(cuda_check(cudaMemsetAsync(a->umap, 0, (size_t)a->umap_n, st), "unit map clear"));
     a->cur = 0;
     a->steps_done = 0;

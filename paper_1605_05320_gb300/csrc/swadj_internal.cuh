@@ -24,6 +24,34 @@ struct DevClock {
     double smax;        // s_max(Q^n)
 };
 
+// Marks of the units of an FP32 2D step.  STILL: every cell of the unit is
+// zero in both buffers.  A unit that is still among still neighbours has a
+// still window (a unit's window reaches less than one unit beyond it, and
+// ghost cells are cells of the units at the boundary), stays so, and needs
+// neither its scan nor its stores.
+enum : unsigned char {
+    UNIT_UNKNOWN = 0,
+    UNIT_ACTIVE = 1,   // it had waves at an earlier step and is not scanned again
+    UNIT_STILL = 2
+};
+
+// Whether every unit around unit (sx, sy) of an nsx x nsy map, itself
+// included, is still; own: its mark.  Called by a whole warp.  A neighbour
+// that turns active in this very step still has still cells at its start, so
+// it does not matter which of its two marks is seen.
+__device__ __forceinline__ bool still_around(const unsigned char *map, int sx, int sy, int nsx,
+                                             int nsy, int &own) {
+    const int lane = threadIdx.x & 31;
+    const int dx = lane & 3, dy = lane >> 2;   // lanes 0-2, 4-6, 8-10
+    int m = UNIT_STILL;
+    if (dx < 3 && dy < 3) {
+        const int x = sx + dx - 1, y = sy + dy - 1;
+        if (x >= 0 && x < nsx && y >= 0 && y < nsy) m = map[(size_t)y * nsx + x];
+    }
+    own = __shfl_sync(0xffffffffu, m, 5);
+    return __all_sync(0xffffffffu, m == UNIT_STILL);
+}
+
 // Bits set in the device error word.
 enum : int {
     ERR_UNSTABLE = 1,   // non-finite state or depth <= 0
