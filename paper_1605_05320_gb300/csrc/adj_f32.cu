@@ -213,8 +213,9 @@ __global__ void __launch_bounds__(256, 4) adj_f32_strips(AdjParams<float> p, int
     // and late in the zero phase: 2048^2 17.5 / 10.5 and 34.2 / 29.5, 4096^2
     // 68 / 13 and 76 / 36.  Where most units are active the nine marks cost
     // what they save: 512^2 5.9 / 6.1, 1024^2 8.0 / 6.9 and 12.8 / 13.0.
-    int own = UNIT_ACTIVE;
-    const bool still = p.umap && still_around(p.umap, sx, sy, nsx, nsy, own);
+    const int own = p.umap ? p.umap[unit] : (int)UNIT_ACTIVE;
+    const bool still = own == UNIT_STILL &&
+                       still_around(p.umap, unit, sx, nsx, nsx * nsy, UNIT_STILL);
     if (still && !p.snap_f && !p.snap_d) return;
     const bool scan = own != UNIT_ACTIVE;
     if (still || (scan && quiet_a(p, col, y0, ylast, yin))) {   // quiet: the unit stays zero

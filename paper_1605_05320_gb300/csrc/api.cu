@@ -207,7 +207,7 @@ struct swa_grid {
     long long *gauge_row;  // device row counter of the fused gauge recording
     GaugeRec gauges;       // fused gauge recording (n = 0: off)
     float *rest_tab;       // FP32 2D: rest CFL table of the step's quiet units
-    unsigned char *umap;   // FP32 2D: units that have had waves (quiet-unit hint)
+    unsigned char *umap;   // FP32 2D: marks of the step's units
     int umap_n;
 };
 
@@ -296,6 +296,8 @@ int swadj::grid_refs(const swa_grid *g, GridRefs *out) {
     out->clk = g->clk;
     out->state_set = g->state_set;
     out->scheme = g->scheme;
+    out->umap = g->umap;
+    out->umap_n = g->umap_n;
     return SWA_OK;
 }
 

@@ -23,7 +23,7 @@ struct FwdParams {
     int fwd_rows;      // FP32 strip height (rows per block), 0 = default
     int keep_rest;     // FP32 2D: 1 computes wave-free rows in full (no skipping)
     const float *rest_tab;   // FP32 2D grid: rest CFL table of quiet units (null: none)
-    unsigned char *umap;     // FP32 2D grid: 1 = unit had waves at an earlier step
+    unsigned char *umap;     // FP32 2D grid: marks of the strip step's units
     int umap_n;              // entries of umap
     GaugeRec gauges;   // fused gauge recording (n = 0: off)
     int keep_input;    // FP64 2D: 1 leaves the old state in place and writes the other buffer

@@ -55,10 +55,18 @@ __global__ void __launch_bounds__(strip::kThreads, 4)
     bool bad = false;
     const int lane = threadIdx.x & 31;
     const bool quiet = p.rest_tab && p.umap && !p.keep_rest;
+    // Marks carry the unit height: those of another one (the caller may change
+    // it, and a captured step keeps its own) say nothing.
+    const int tag = (rows & 63) << 2;
+    // the first unit by position, the others from the counter (the counter's
+    // first round trip cost 1.1 us of 15.5 at 512^2)
+    int next = lane == 0 ? (int)(blockIdx.x * (strip::kThreads / 32) + (threadIdx.x >> 5)) : -1;
     for (;;) {   // warp-uniform
-        int u = 0;
-        if (lane == 0) u = (int)atomicAdd(&p.clk->work, 1u);
+        int u = next;
+        if (lane == 0 && u < 0)
+            u = (int)(gridDim.x * (strip::kThreads / 32) + atomicAdd(&p.clk->work, 1u));
         u = __shfl_sync(0xffffffffu, u, 0);
+        next = -1;
         if (u >= nunits) {
             if (u >= nunits + ngroups) break;
             record_gauge_group<float>(p.gauges, p.q[cur][0], p.bath, p.nx, p.ny, 1, p.clk,
@@ -66,14 +74,30 @@ __global__ void __launch_bounds__(strip::kThreads, 4)
             continue;
         }
         const int sy = u / nsx, sx = u - sy * nsx;
-        // A unit that had waves at an earlier step keeps them (the ocean does
-        // not return exactly to rest behind a wave): it skips the quiet scan.
-        // The map is only a hint; the scan alone decides that a unit is quiet.
-        if (quiet && (u >= p.umap_n || p.umap[u] == 0)) {
-            if (strip::quiet_unit<true>(v, p.rest_tab, sx, sx * strip::kOut, sy * rows, rows, p.g,
-                                        smax))
-                continue;
-            if (lane == 0 && u < p.umap_n) p.umap[u] = 1;
+        if (quiet) {
+            const int own = p.umap[u];
+            if (own != (tag | UNIT_ACTIVE)) {
+                // still among still units: both buffers hold it at rest, and
+                // only its CFL terms count (2048^2 at rest but for a small
+                // source 35 us with each unit scanned and stored, 29 so;
+                // 4096^2 81 and 44)
+                if (own == (tag | UNIT_STILL) &&
+                    still_around(p.umap, u, sx, nsx, nunits, tag | UNIT_STILL)) {
+                    const int yend = (sy + 1) * rows < p.ny ? (sy + 1) * rows : p.ny;
+                    for (int j = sy * rows + lane; j < yend; j += 32)
+                        smax = fmaxf(smax, p.rest_tab[(size_t)sx * p.ny + j]);
+                    continue;
+                }
+                // the scan alone decides that a unit is at rest; one that has
+                // had waves keeps them (the ocean does not return exactly to
+                // rest behind a wave) and is not scanned again
+                if (strip::quiet_unit<true>(v, p.rest_tab, sx, sx * strip::kOut, sy * rows, rows,
+                                            p.g, smax)) {
+                    if (lane == 0) p.umap[u] = tag | UNIT_STILL;
+                    continue;
+                }
+                if (lane == 0) p.umap[u] = tag | UNIT_ACTIVE;
+            }
         }
         // Units with waves take the full path: quiet units cover the ocean
         // at rest, and the strip loop without its row skipping is leaner.
@@ -84,6 +108,12 @@ __global__ void __launch_bounds__(strip::kThreads, 4)
             strip::strip_unit<ORD, 2>(v, sx * strip::kOut, sy * rows, rows, s_nu[0], s_nu[1], p.g,
                                       ring[threadIdx.x >> 5], smax, bad);
     }
+    // no marks but this step's units': without this, heights changed to and
+    // fro would find old marks where the other height has fewer units
+    if (p.umap)
+        for (int k = (quiet ? nunits : 0) + blockIdx.x * strip::kThreads + threadIdx.x;
+             k < p.umap_n; k += gridDim.x * strip::kThreads)
+            p.umap[k] = UNIT_UNKNOWN;
     if (bad) atomicOr(p.err, ERR_UNSTABLE);
     fwave::finish_step<strip::kThreads>(p.clk, p.partial, p.nblocks, p.cfl, smax, red, &am_last,
                                         t_now, dt, cur);

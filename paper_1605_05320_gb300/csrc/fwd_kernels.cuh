@@ -204,6 +204,10 @@ fwd_step_kernel(FwdParams<R> p) {
     const int cur = clk->cur;
     if (p.gauges.n > 0 && blockIdx.x == 0 && blockIdx.y == 0)   // the state this step starts from
         record_gauges<R, NT>(p.gauges, p.q[cur][0], p.bath, p.nx, p.ny, p.two_d, t);
+    // the marks of the strip step's units do not hold after this step
+    if (p.umap && blockIdx.x == 0)
+        for (int k = blockIdx.y * NT + tid; k < p.umap_n; k += gridDim.y * NT)
+            p.umap[k] = UNIT_UNKNOWN;
 
     const R *q0 = p.q[cur][0], *q1 = p.q[cur][1], *q2 = p.q[cur][2];
     R *o0 = p.q[cur ^ 1][0], *o1 = p.q[cur ^ 1][1], *o2 = p.q[cur ^ 1][2];
@@ -453,7 +457,7 @@ __global__ void __launch_bounds__(256) clock_init_kernel(FwdParams<R> p, double 
     const int tid = threadIdx.x;
     const size_t n = (size_t)p.nx * p.ny;
     R *q0 = p.q[0][0], *q1 = p.q[0][1], *q2 = p.q[0][2];
-    // a new state: no unit has had waves yet (the quiet-unit hint)
+    // a new state: nothing is known of the strip step's units
     for (int k = blockIdx.x * 256 + tid; k < p.umap_n; k += gridDim.x * 256) p.umap[k] = 0;
     // maxima of the CFL number (float rule), or of |u| + c and |v| + c, whose
     // divisions by dx and dy wait for the end (they are monotone)

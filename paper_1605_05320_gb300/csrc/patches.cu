@@ -1006,6 +1006,8 @@ struct AvgParams {
     double *slot;                  // 1 + r per edge
     double t_end;                  // the parent's step end
     int *err;
+    unsigned char *umap;           // the unit marks of the coarse grid's step,
+    int umap_n;                    // where it is the parent: its state changes
 };
 
 // Every copy of a parent cell under the level := mean of its r x r cells
@@ -1049,6 +1051,9 @@ __global__ void amr_avg_kernel(AvgParams p) {
         float *dst = (m.x < 0 ? *p.coarse : p.table[m.x]).q[pcur][k];
         dst[m.y] = block_sum<R>(S.q[fcur][k] + m.w, S.nx, r) * inv;
     }
+    // a unit at rest may have waves now; one that had waves stays marked
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < p.umap_n; k += gridDim.x * blockDim.x)
+        if (p.umap[k] & UNIT_STILL) p.umap[k] = UNIT_UNKNOWN;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const double tol = 1e-12 * (fabs(p.t_end) > 1.0 ? fabs(p.t_end) : 1.0);
         if (!(fabs(lc->t - p.t_end) <= tol) || !(fabs(pc->t - p.t_end) <= tol))
@@ -1389,6 +1394,7 @@ int amr_average(swa_amr *A, const GridRefs &c, int l, double t_end, bool reflux,
     p.slot = V.slot;
     p.t_end = t_end;
     p.err = swadj_host::error_word();
+    if (l == 1) { p.umap = c.umap; p.umap_n = c.umap_n; }
     const size_t n = (size_t)3 * V.navg + (size_t)p.ncfu;
     const unsigned ab = patches::ew_blocks(n > 0 ? n : 1);
     void (*kernel)(amr::AvgParams) = amr::amr_avg_kernel<0>;

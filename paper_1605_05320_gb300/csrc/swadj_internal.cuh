@@ -24,32 +24,32 @@ struct DevClock {
     double smax;        // s_max(Q^n)
 };
 
-// Marks of the units of an FP32 2D step.  STILL: every cell of the unit is
-// zero in both buffers.  A unit that is still among still neighbours has a
-// still window (a unit's window reaches less than one unit beyond it, and
-// ghost cells are cells of the units at the boundary), stays so, and needs
-// neither its scan nor its stores.
+// Marks of the units of the FP32 2D steps (the forward step's, which adds the
+// unit height above the two lowest bits, and the adjoint's).  STILL: every cell of the unit is zero (at rest) in both
+// buffers.  A unit that is still among still neighbours has a still window
+// (a unit's window reaches less than one unit beyond it, and ghost cells are
+// cells of the units at the boundary), stays so, and needs neither its scan
+// nor its stores.
 enum : unsigned char {
     UNIT_UNKNOWN = 0,
     UNIT_ACTIVE = 1,   // it had waves at an earlier step and is not scanned again
     UNIT_STILL = 2
 };
 
-// Whether every unit around unit (sx, sy) of an nsx x nsy map, itself
-// included, is still; own: its mark.  Called by a whole warp.  A neighbour
-// that turns active in this very step still has still cells at its start, so
-// it does not matter which of its two marks is seen.
-__device__ __forceinline__ bool still_around(const unsigned char *map, int sx, int sy, int nsx,
-                                             int nsy, int &own) {
+// Whether the units around unit u (column sx of a map of nsx columns and n
+// units), itself included, all carry `mark`, that of a still unit.  Called by
+// a whole warp.  A neighbour that turns active in this very step still has
+// still cells at its start, so it does not matter which of its two marks is
+// seen.  Asked for still units only: the active ones, which take the time,
+// read their own mark and no more.
+__device__ __forceinline__ bool still_around(const unsigned char *map, int u, int sx, int nsx,
+                                             int n, int mark) {
     const int lane = threadIdx.x & 31;
-    const int dx = lane & 3, dy = lane >> 2;   // lanes 0-2, 4-6, 8-10
-    int m = UNIT_STILL;
-    if (dx < 3 && dy < 3) {
-        const int x = sx + dx - 1, y = sy + dy - 1;
-        if (x >= 0 && x < nsx && y >= 0 && y < nsy) m = map[(size_t)y * nsx + x];
-    }
-    own = __shfl_sync(0xffffffffu, m, 5);
-    return __all_sync(0xffffffffu, m == UNIT_STILL);
+    const int dx = (lane & 3) - 1, dy = (lane >> 2) - 1;   // lanes 0-2, 4-6, 8-10
+    const int x = sx + dx, k = u + dy * nsx;
+    bool ok = true;
+    if (dx < 2 && dy < 2 && x >= 0 && x < nsx && k >= 0 && k < n) ok = map[k + dx] == mark;
+    return __all_sync(0xffffffffu, ok);
 }
 
 // Bits set in the device error word.
@@ -166,6 +166,8 @@ struct GridRefs {
     DevClock *clk;
     int state_set;
     int scheme;         // SWA_SCHEME_SPLIT or SWA_SCHEME_CTU
+    unsigned char *umap;   // FP32 2D: the step's unit marks, cleared when the
+    int umap_n;            // state is written by anything but a strip step
 };
 int grid_refs(const swa_grid *g, GridRefs *out);
 // FP64 mass audit (audit.cu)
