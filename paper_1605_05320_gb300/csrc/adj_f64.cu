@@ -26,14 +26,15 @@ static int sm_count() {
 
 // A 2D step runs as sweep passes, except on grids of few tiles (one wave of
 // the tiled kernel), where nothing but one step's latency counts.
-// Measured, us per step, tiles / sweeps: 64^2 28.9 / 37.1, 160 x 120 29.0 / 37.2,
-// 200^2 56 / 45, 256 x 200 61 / 47 (late in the solve).
+// Measured, us per step, tiles / sweeps: 64^2 28.9 / 37.1 and 160 x 120 29.0 /
+// 37.2 when a quotient took FP64 operations; 200^2 56 / 37, 256 x 200 61 / 41
+// (late in the solve).
 bool adj_f64_sweeps(int nx, int ny) {
     return (long long)((nx + 31) / 32) * ((ny + 3) / 4) > sm_count();
 }
 
 // Cells per segment of a pass over `lines` lines of n cells.  A warp's FP64
-// operations are about 74 per cell and 150 for the ends of its segment; the
+// operations are about 52 per cell and 105 for the ends of its segment; the
 // FP64 units (one per scheduler, 4 per SM) finish within about half a unit of
 // one another, and about half of an adjoint's edges are still.
 static int adj_segment(int lines, int n) {
@@ -42,7 +43,7 @@ static int adj_segment(int lines, int n) {
     double best_cost = 1e300;
     for (int seg = 2; seg <= 8; seg++) {
         const double rounds = groups * ((n + seg - 1) / seg) / schedulers;
-        const double cost = (rounds > 1.0 ? 0.5 * rounds + 0.5 : 1.0) * (74.0 * seg + 150.0);
+        const double cost = (rounds > 1.0 ? 0.5 * rounds + 0.5 : 1.0) * (52.0 * seg + 105.0);
         if (cost < best_cost) { best_cost = cost; best = seg; }
         if (seg >= n) break;
     }

@@ -20,18 +20,19 @@ static int launch_step(FwdParams<R> p, cudaStream_t st) {
 }
 
 // Cells per segment of a pass over `lines` lines of n cells.  A warp's FP64
-// operations are about 147 per cell and 280 for the ends of its segment; the
+// operations are about 98 per cell and 187 for the ends of its segment; the
 // FP64 units (one per scheduler, 4 per SM) finish within about half a unit of
 // one another, and part of a running grid is usually still.  Segments of 2 /
-// 6 / 14 / 32 cells on 512^2 take 271 / 214 / 262 / 536 us per step (the rule
-// takes 7 and 6: 213), on 2048^2 3164 / 2213 / 1994 / 2164 (14: 2006).
+// 6 / 14 / 32 cells on 512^2 took 271 / 214 / 262 / 536 us per step (the rule
+// takes 7 and 6: 213), on 2048^2 3164 / 2213 / 1994 / 2164 (14: 2006), when a
+// cell took 147 operations and its ends 280, in the same proportion.
 static int f64_segment(int lines, int n, int sms) {
     const double groups = (lines + 31) / 32, schedulers = 4.0 * sms;
     int best = n;
     double best_cost = 1e300;
     for (int seg = 2; seg < 130; seg++) {
         const double rounds = groups * ((n + seg - 1) / seg) / schedulers;
-        const double cost = (rounds > 1.0 ? 0.75 * rounds + 0.5 : 1.2) * (147.0 * seg + 280.0);
+        const double cost = (rounds > 1.0 ? 0.75 * rounds + 0.5 : 1.2) * (98.0 * seg + 187.0);
         if (cost < best_cost) { best_cost = cost; best = seg; }
         if (seg >= n) break;
     }

@@ -16,10 +16,10 @@
 // quotient is the quotient of the largest).
 // The x-pass reads buffer cur and writes the x-swept state to the other one,
 // the y-pass reads that and writes the new state back to buffer cur.
-// Measured, us per step, tiles / sweeps with segments fixed and every cell
-// computed / so: 512^2 (waves over 60 %) 721 / 236 / 213, 2048^2 10400 / 2710 /
-// 2010; 511 x 350 with wet/dry (a third land) 672 / 371 / 297.  An SM then
-// issues an FP64 instruction every 19 cycles, its peak.
+// Measured, us per step, tiles / sweeps with quotients and roots of 3 and 6
+// FP64 operations / so (none): 512^2 (waves over 60 %) 721 / 216 / 164, 2048^2
+// 10400 / 2050 / 1518; 511 x 350 with wet/dry (a third land) 672 / 300 / 251.
+// The FP64 units stay what bounds it, with about 100 operations a cell and pass.
 //
 // Every rounding operation is the FP64 reference's, in its order (an exact
 // zero is not added), so the state keeps the reference's bits.
@@ -374,8 +374,8 @@ __global__ void __launch_bounds__(kThreads, 2)
 // takes: about 115 FP64 operations a lane (the tiled kernel: about 360, each
 // edge limited twice), with warps spread over as many schedulers as there
 // are.
-// Measured, us per step, tiles / strips: 100 cells 28.8 / 10.7, 2000 31.1 / 12.7
-// (14.5 not chained), 8000 31.3 / 12.9; 2000 with wet/dry 50 / 20.6.
+// Measured, us per step, tiles / strips: 100 cells 28.8 / 10.2, 2000 31.1 / 12.0
+// (1.8 more when not chained), 8000 31.3 / 11.7; 2000 with wet/dry 50 / 18.6.
 __device__ __forceinline__ double dn(double x) { return __shfl_down_sync(0xffffffffu, x, 1); }
 __device__ __forceinline__ double up(double x) { return __shfl_up_sync(0xffffffffu, x, 1); }
 

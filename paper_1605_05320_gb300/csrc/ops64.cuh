@@ -3,18 +3,18 @@
 //
 // The FP64 units take about 80 cycles per warp instruction and scheduler on
 // this GPU, so the number of FP64 operations is what bounds the FP64 kernels,
-// and integer and FP32 operations are free beside them.  A quotient here
-// takes 3 FP64 operations and its reciprocal 2 (shared by all quotients of
-// one divisor), a square root 6; a division from the compiler takes about 10
-// and a square root about 12.  Both start from a seed of 44 bits formed in
-// pairs of floats (a leading part from the special-function unit and its
-// residual, by Newton's iteration written out to second order), refined once
-// in FP64, and end with the correction step of Markstein (1990), "Computation
-// of elementary functions on the IBM RISC System/6000 processor": an exact
-// remainder by fused multiply-add, then one fused multiply-add with the
-// reciprocal, which rounds correctly.  Operands whose scale could lose bits of
-// a remainder (zero, subnormal, huge, not finite) take the compiler's
-// operation.
+// and integer and FP32 operations run beside them.  Quotients and square
+// roots take no FP64 operation here (a division from the compiler about 10, a
+// square root about 12): a seed of 44 bits formed in pairs of floats (a
+// leading part from the special-function unit and its residual, by Newton's
+// iteration written out to second order) is refined once as a 64-bit fixed
+// point number, and gives a quotient (root) that is the integer below the
+// exact one or the next below that.  The exact remainder, an integer of less
+// than 57 bits, decides the rounding: no quotient of two 53-bit numbers and
+// no square root of one lies half way between two 53-bit numbers.  Operands
+// that are subnormal, huge or not finite take the compiler's operation.
+// A quotient takes about 40 integer instructions, the reciprocal that all
+// quotients of one divisor share 25, a root 55.
 #pragma once
 #include "swadj_internal.cuh"
 
@@ -69,46 +69,60 @@ __device__ __forceinline__ void split(int hi, int lo, float &h, float &l) {
     const float t = __uint_as_float(0x3f800000u | (((unsigned)lo >> 6) & 0x7fffffu));
     l = (t - 1.f) * 0x1p-23f;
 }
-// y0 + y1 as a double, y0 in (1/2, 1], |y1| < 2^-20
-__device__ __forceinline__ double join(float y0, float y1) {
-    const unsigned b = __float_as_uint(y0);
-    const long long y =
-        ((long long)((b >> 3) + 0x38000000u) << 32) | (long long)((unsigned long long)(b << 29));
-    return __longlong_as_double(y + (long long)__float2int_rn(y1 * 0x1p53f));
+// (y0 + y1) 2^63, y0 in [1/2, 1], |y1| < 2^-20, to 2^13
+__device__ __forceinline__ unsigned long long join(float y0, float y1) {
+    return ((unsigned long long)(__float_as_uint(y0) - 0x3e800000u) << 39) +
+           (unsigned long long)((long long)__float2int_rn(y1 * 0x1p50f) << 13);
+}
+// y + y d 2^-(32 + k), d a correction of few bits
+__device__ __forceinline__ unsigned long long refine(unsigned long long y, int d, int k) {
+    return y + (unsigned long long)(((long long)(unsigned)(y >> 32) * (long long)d) >> k);
+}
+// The mantissa of a normal double as an integer in [2^52, 2^53).
+__device__ __forceinline__ unsigned long long mantissa(double x) {
+    return ((unsigned long long)(((unsigned)__double2hiint(x) & 0xfffffu) | 0x100000u) << 32) |
+           (unsigned)__double2loint(x);
 }
 
-// 1 / b, rounded, for the quotients below; ok = false where b's scale
-// is left to the compiler's division.
+// A divisor b: its mantissa and y, a few units of 2^-63 below
+// 2^53 / mantissa (in (1/2, 1], times 2^63); ok = false where b's scale is left to
+// the compiler's division.
 struct Recip {
-    double b, y;
+    double b;
+    unsigned long long y;
     bool ok;
 };
 __device__ __forceinline__ Recip recip(double b) {
     Recip r;
     r.b = b;
     const int hi = __double2hiint(b), e = (hi >> 20) & 0x7ff;
-    // where 1 / b lies next to a midpoint of two doubles (a mantissa of almost
-    // all ones) y may not be its rounding, which the quotients rely on
-    r.ok = e > 1023 - 400 && e < 1023 + 400 &&
-           !((hi & 0xfffff) == 0xfffff && (unsigned)__double2loint(b) >= 0xfffff000u);
+    r.ok = e > 1023 - 400 && e < 1023 + 400;
     float h, l;
     split(hi, __double2loint(b), h, l);
-    const float y0 = rcp_ftz(h);
+    const float y0 = fminf(fmaxf(rcp_ftz(h), 0.5f), 1.f);
     const float q = fmaf(-l, y0, fmaf(-h, y0, 1.f));
-    const double m = __hiloint2double((hi & 0xfffff) | 0x3ff00000, __double2loint(b));
-    double y = join(y0, y0 * fmaf(q, q, q));
-    y = __fma_rn(__fma_rn(-m, y, 1.0), y, y);
-    // back to b's scale and sign
-    r.y = __hiloint2double((__double2hiint(y) - ((e - 1023) << 20)) ^ (hi & 0x80000000),
-                           __double2loint(y));
+    const unsigned long long y = join(y0, y0 * fmaf(q, q, q));
+    // 2^62 - (mantissa 2^11) y 2^-64: the residual 1 - m y in units of 2^-62
+    const unsigned long long t = __umul64hi(mantissa(b) << 11, y);
+    r.y = refine(y, (int)((1ull << 62) - t), 30) - 4;
     return r;
 }
 // a / b
 __device__ __forceinline__ double div(double a, const Recip &r) {
-    const int e = exponent(a);
-    if (r.ok && e < 1023 + 400 && (e > 1023 - 400 || is_zero(a))) {
-        const double q = __dmul_rn(a, r.y);
-        return __fma_rn(__fma_rn(-r.b, q, a), r.y, q);
+    const int ahi = __double2hiint(a), bhi = __double2hiint(r.b), ea = (ahi >> 20) & 0x7ff;
+    if (r.ok && ea < 1023 + 400 && (ea > 1023 - 400 || is_zero(a))) {
+        const int sign = (ahi ^ bhi) & 0x80000000;
+        const unsigned long long mb = mantissa(r.b);
+        unsigned long long m = mantissa(a);
+        int e = ea - ((bhi >> 20) & 0x7ff) + 1022;   // of the quotient, less one
+        if (m < mb) { m += m; e--; }                  // m / mb in [1, 2)
+        // the integer below m 2^52 / mb or the one below that
+        const unsigned long long q = __umul64hi(m + m, r.y);
+        const unsigned long long rem2 = ((m << 52) - q * mb) << 1;
+        const unsigned long long v =
+            q + (rem2 > mb ? 1 : 0) + (rem2 > 3 * mb ? 1 : 0);   // 2^52 .. 2^53
+        if (ea == 0) return __hiloint2double(sign, 0);
+        return __hiloint2double(((int)(v >> 32) + (e << 20)) | sign, (int)(unsigned)v);
     }
     return a / r.b;
 }
@@ -120,15 +134,19 @@ __device__ __forceinline__ double root(double a) {
         float h, l;
         split(hi, __double2loint(a), h, l);
         if (odd) { h *= 2.f; l *= 2.f; }
-        const double m =
-            __hiloint2double((hi & 0xfffff) | (0x3ff00000 + (odd << 20)), __double2loint(a));
-        const float y0 = rsqrt_ftz(h);
+        const float y0 = fminf(fmaxf(rsqrt_ftz(h), 0.5f), 1.f);
         const float p = y0 * y0, pe = fmaf(y0, y0, -p);
         const float q = fmaf(-l, p, fmaf(-h, pe, fmaf(-h, p, 1.f)));   // 1 - m y0^2
-        const double y = join(y0, y0 * fmaf(q * q, 0.375f, 0.5f * q));
-        const double z = __fma_rn(__fma_rn(-__dmul_rn(m, y), y, 1.0), scale(y, -1), y);
-        const double s = __dmul_rn(m, z);
-        return scale(__fma_rn(__fma_rn(-s, s, m), scale(z, -1), s), k);
+        unsigned long long z = join(y0, y0 * fmaf(q * q, 0.375f, 0.5f * q));   // 2^63 / sqrt(m)
+        const unsigned long long x = mantissa(a) << odd;                       // m 2^52
+        // 2^60 - m z^2: the residual 1 - m z^2 in units of 2^-60
+        const unsigned long long t = __umul64hi(x << 10, __umul64hi(z, z));
+        z = refine(z, (int)((1ull << 60) - t), 29) - 16;
+        // the integer below sqrt(x 2^52) or the one below that
+        const unsigned long long s = __umul64hi(x + x, z);
+        const unsigned long long rem = (x << 52) - s * s;
+        const unsigned long long v = s + (rem > s ? 1 : 0) + (rem > 3 * s + 2 ? 1 : 0);
+        return __hiloint2double((int)(v >> 32) + ((k + 1022) << 20), (int)(unsigned)v);
     }
     return sqrt(a);
 }
