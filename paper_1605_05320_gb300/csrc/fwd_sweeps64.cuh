@@ -17,9 +17,10 @@
 // The x-pass reads buffer cur and writes the x-swept state to the other one,
 // the y-pass reads that and writes the new state back to buffer cur.
 // Measured, us per step, tiles / sweeps with quotients and roots of 3 and 6
-// FP64 operations / so (none): 512^2 (waves over 60 %) 721 / 216 / 164, 2048^2
-// 10400 / 2050 / 1518; 511 x 350 with wet/dry (a third land) 672 / 300 / 251.
-// The FP64 units stay what bounds it, with about 100 operations a cell and pass.
+// FP64 operations / so (none): 512^2 (waves over 60 %) 721 / 216 / 160, 2048^2
+// 10400 / 2050 / 1462; 511 x 350 with wet/dry (a third land) 672 / 300 / 242.
+// The FP64 units stay what bounds it, with about 95 operations a cell and pass
+// (the cell's products formed once, not for both its edges: 3 % of it).
 //
 // Every rounding operation is the FP64 reference's, in its order (an exact
 // zero is not added), so the state keeps the reference's bits.
@@ -36,6 +37,7 @@ using namespace d64;
 // A cell in the frame of a sweep (mn the momentum normal to the edges).
 struct Cell {
     double h, mn, mt, eta, un, ut, sq, b;
+    double fn, ft, wn, wt;   // mn un, mn ut and sq un, sq ut, one product for both edges
 };
 
 // A solved edge: wave speeds, the vectors of waves 1 and 3, the strength of
@@ -54,11 +56,16 @@ __device__ __forceinline__ Cell derive(double tol, double h, double mn, double m
     Cell c;
     c.h = h; c.mn = mn; c.mt = mt; c.eta = eta; c.b = b;
     c.un = 0.0; c.ut = 0.0; c.sq = 0.0;
+    c.fn = 0.0; c.ft = 0.0; c.wn = 0.0; c.wt = 0.0;
     if (moving && (!WD || h > tol)) {
         const Recip r = recip(h);
         c.un = div(mn, r);
         c.ut = div(mt, r);
         c.sq = root(h);
+        c.fn = mn * c.un;
+        c.ft = mn * c.ut;
+        c.wn = c.sq * c.un;
+        c.wt = c.sq * c.ut;
     }
     return c;
 }
@@ -109,8 +116,8 @@ __device__ __forceinline__ void shore(double g, const Cell &L, const Cell &R, do
             else F[m] = div(sR * FL[m] - sL * FR[m] + sL * sR * (QR[m] - QL[m]), w);
         }
     }
-    const double fL[3] = {L.mn, L.mn * L.un + pL, L.mn * L.ut};
-    const double fR[3] = {R.mn, R.mn * R.un + pR, R.mn * R.ut};
+    const double fL[3] = {L.mn, L.fn + pL, L.ft};
+    const double fR[3] = {R.mn, R.fn + pR, R.ft};
     am[0] = F[0] - fL[0]; am[1] = (F[1] + (pL - pLs)) - fL[1]; am[2] = F[2] - fL[2];
     ap[0] = fR[0] - F[0]; ap[1] = fR[1] - (F[1] + (pR - pRs)); ap[2] = fR[2] - F[2];
 }
@@ -141,13 +148,13 @@ __device__ __forceinline__ Edge solve(double g, double tol, const Cell &L, const
     }
     const double gh = g * half_of(L.h + R.h);
     const Recip den = recip(L.sq + R.sq);
-    const double uh = div(L.sq * L.un + R.sq * R.un, den);
-    const double vh = div(L.sq * L.ut + R.sq * R.ut, den);
+    const double uh = div(L.wn + R.wn, den);
+    const double vh = div(L.wt + R.wt, den);
     const double ch = root(gh);
     e.s1 = uh - ch; e.s2 = uh; e.s3 = uh + ch;
     const double df1 = R.mn - L.mn;
-    const double df2 = (R.mn * R.un - L.mn * L.un) + gh * (R.eta - L.eta);
-    const double df3 = R.mn * R.ut - L.mn * L.ut;
+    const double df2 = (R.fn - L.fn) + gh * (R.eta - L.eta);
+    const double df3 = R.ft - L.ft;
     const Recip w = recip(e.s3 - e.s1);
     const double b1 = div(e.s3 * df1 - df2, w), b3 = div(df2 - e.s1 * df1, w);
     e.b2 = df3 - vh * df1;
@@ -409,6 +416,7 @@ __global__ void __launch_bounds__(32) fwd_f64_line(FwdParams<double> p) {
         Cell r;
         r.h = dn(c.h); r.mn = dn(c.mn); r.mt = 0.0; r.eta = dn(c.eta); r.un = dn(c.un);
         r.ut = 0.0; r.sq = dn(c.sq); r.b = dn(c.b);
+        r.fn = dn(c.fn); r.wn = dn(c.wn); r.ft = 0.0; r.wt = 0.0;
         const bool still = __all_sync(0xffffffffu, is_still<WD>(tol, c, r));
         Edge w = {};
         if (!still) w = solve<WD>(g, tol, c, r);   // edge (i|i+1)
