@@ -444,12 +444,19 @@ fwd_step_kernel(FwdParams<R> p) {
     }
 }
 
+template <typename R>
+__device__ __forceinline__ R from_double(double x) { return (R)x; }
+template <>
+__device__ __forceinline__ float from_double<float>(double x) { return d64::to_float(x); }
+
 // Initial CFL reduction over buffer 0 (set_state), same per-cell rule.  SET:
 // the buffer is set first, cell by cell, from FP64 arrays on the device
 // (surface elevation and momenta; PERT keeps eta, else h = eta - B), so a
 // state set from the device is one pass over memory.
 // Measured on 2048^2 FP32: 28 us for the reduction and 42 us for the three
-// conversions and the clear before it, 50 us for both in one.
+// conversions and the clear before it, 50 us for both in one, 40 without FP64
+// operations (4096^2 179 / 142 us a call): three conversions, and the maximum
+// kept as a float.  167 MB pass through memory.
 template <typename R, bool PERT, bool SET>
 __global__ void __launch_bounds__(256) clock_init_kernel(FwdParams<R> p, double t0, StateSrc src) {
     __shared__ double red[32];
@@ -462,14 +469,16 @@ __global__ void __launch_bounds__(256) clock_init_kernel(FwdParams<R> p, double 
     // maxima of the CFL number (float rule), or of |u| + c and |v| + c, whose
     // divisions by dx and dy wait for the end (they are monotone)
     double mx = 0.0, my = 0.0;
+    float smax = 0.f;
+    const float rdx = 1.f / (float)p.dx, rdy = 1.f / (float)p.dy;
     for (size_t k = (size_t)blockIdx.x * 256 + tid; k < n; k += (size_t)gridDim.x * 256) {
         const R b = p.bath[k];
         R a, u, v;
         if (SET) {
             const double eta = src.eta[k];
-            a = PERT ? (R)eta : (R)(eta - (double)b);
-            u = (R)src.hu[k];
-            v = p.two_d ? (R)src.hv[k] : R(0);
+            a = PERT ? from_double<R>(eta) : (R)(eta - (double)b);
+            u = from_double<R>(src.hu[k]);
+            v = p.two_d ? from_double<R>(src.hv[k]) : R(0);
             q0[k] = a;
             q1[k] = u;
             q2[k] = v;
@@ -485,9 +494,8 @@ __global__ void __launch_bounds__(256) clock_init_kernel(FwdParams<R> p, double 
         }
         if (PERT) {
             // the float rule of the fused step reduction (cfl_f32)
-            const double sd = (double)cfl_f32((float)h, (float)u, (float)v, (float)p.g,
-                                              1.f / (float)p.dx, 1.f / (float)p.dy, p.two_d);
-            mx = sd > mx ? sd : mx;
+            smax = fmaxf(smax, cfl_f32((float)h, (float)u, (float)v, (float)p.g, rdx, rdy,
+                                       p.two_d));
         } else {
             const d64::Recip r = d64::recip((double)h);
             const double c = d64::root((double)(p.g * h));
@@ -502,7 +510,9 @@ __global__ void __launch_bounds__(256) clock_init_kernel(FwdParams<R> p, double 
         }
         if (p.err && !(h > R(0))) atomicOr(p.err, ERR_UNSTABLE);
     }
-    if (!PERT) {
+    if (PERT) {
+        mx = (double)smax;
+    } else {
         mx = mx / (double)p.dx;
         my = my / (double)p.dy;
         mx = my > mx ? my : mx;

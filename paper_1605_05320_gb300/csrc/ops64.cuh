@@ -62,6 +62,21 @@ __device__ __forceinline__ bool is_nan(double x) {
     return (__double_as_longlong(x) & 0x7fffffffffffffffLL) > 0x7ff0000000000000LL;
 }
 
+// (float)x, to nearest even.  The hardware's conversion goes through the FP64
+// units, which bound the kernel that sets an FP32 state from FP64 arrays.
+__device__ __forceinline__ float to_float(double x) {
+    const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+    const unsigned lo = (unsigned)__double2loint(x), sign = (unsigned)hi & 0x80000000u;
+    if (e >= 897 && e <= 1150) {   // from the smallest normal float; may round to infinity
+        unsigned b = (((unsigned)hi & 0x7fffffffu) - (896u << 20)) << 3 | lo >> 29;
+        const unsigned rest = lo << 3;   // the bits below, 2^31 one half
+        b += rest > 0x80000000u || (rest == 0x80000000u && (b & 1));
+        return __uint_as_float(b | sign);
+    }
+    if (is_zero(x)) return __uint_as_float(sign);
+    return (float)x;
+}
+
 // The mantissa (in [1, 2)) of a normal double as a float of its leading 24
 // bits and one of the next 23 (to 2^-47).
 __device__ __forceinline__ void split(int hi, int lo, float &h, float &l) {

@@ -110,3 +110,18 @@ def test_patch_states_on_the_device(S):
         for key, o in zip(("h", "hu", "hv", "eta"), out):
             assert np.array_equal(got[0][1][k][key], got[1][1][k][key])
             assert np.array_equal(o.cpu().numpy(), got[0][1][k][key])
+
+
+def test_conversion_equals_the_hardwares(tmp_path):
+    """Doubles at, beside and between floats and of any bit pattern to float:
+    the hardware's bits."""
+    import os
+    import subprocess
+
+    from paper_1605_05320_gb300 import build as B
+    exe = str(tmp_path / "convert_check")
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "native", "convert_check.cu")
+    subprocess.run([B._nvcc()] + B.NVCC_FLAGS + [src, "-o", exe], check=True,
+                   capture_output=True)
+    r = subprocess.run([exe], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, r.stdout + r.stderr
