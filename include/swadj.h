@@ -147,11 +147,11 @@ int swa_grid_set_strip_rows(swa_grid *grid, int rows);
 
 /*
  * FP32 2D grids: on = 1 (the default) lets the step skip the wave arithmetic
- * of rows that are exactly at rest (eta = hu = hv = 0 across a warp's strip
- * row), where every wave is zero and the exact result is known, and write a
- * strip unit whose whole stencil window is at rest straight back at rest
- * (its CFL terms from a table of the bathymetry's rest terms, formed when
- * the grid is created); on = 0 computes them in full.  Both give the same
+ * of strip units whose whole stencil window is exactly at rest (eta = hu = hv
+ * = 0), where every wave is zero and the exact result is known: such a unit
+ * is written at rest once and left alone while it and its neighbours stay so
+ * (its CFL terms come from a table of the bathymetry's rest terms, formed
+ * when the grid is created); on = 0 computes every unit in full.  Both give the same
  * state and time step (up to the sign of an exact zero); the switch exists
  * to show that and to time the step without the shortcut.  SWA_EINVAL for a
  * null grid or on not 0 or 1.
@@ -197,9 +197,9 @@ int swa_grid_set_scheme(swa_grid *grid, int scheme);
  * against dry land stays exactly at rest, and the mass is conserved between
  * walls as long as no depth goes negative, which the reconstruction
  * guarantees for cfl <= 1/2 (above it a cell that would go negative is set
- * dry, adding its deficit).  The option runs the tiled split kernel (FP64:
- * the reference's rounding; FP32: the perturbation form), not the FP32
- * strip kernel; with SWA_SCHEME_CTU a step returns SWA_EINVAL.  Host state
+ * dry, adding its deficit).  The option runs the sweep passes of the split
+ * step (FP64: the reference's rounding) or its tiled kernel (FP32: the
+ * perturbation form), not the FP32 strip kernel; with SWA_SCHEME_CTU a step returns SWA_EINVAL.  Host state
  * only.
  */
 int swa_grid_set_wetdry(swa_grid *grid, int on);
@@ -302,7 +302,8 @@ int swa_snapstore_info(const swa_snapstore *store, int *count, double *tau_host,
  * and FP32 snapshots of a 2D adjoint grid, the same grid or another one), a
  * snapshot group is read for a cell only if its envelope bound on
  * |q^ . q| reaches tol (1 - 1e-5) there (on another grid: the largest
- * envelope entry over the quads of the cell's bilinear stencil);
+ * envelope entry over the quads of the cell's bilinear stencil; flags_dev
+ * must be aligned to 4 bytes for this, else the full pass runs);
  * the flags and the count are identical to the full pass (every product the
  * pruned pass forms is the one the full pass forms; skipped products are
  * provably below tol), so only the optional m output needs the full pass.

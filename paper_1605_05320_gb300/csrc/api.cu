@@ -201,7 +201,7 @@ struct swa_grid {
     int step_blocks;
     int state_set;
     int strip_rows;        // FP32 launch shape (0 = default)
-    int keep_rest;         // FP32 2D: compute wave-free rows in full
+    int keep_rest;         // FP32 2D: compute units at rest in full
     int scheme;            // 2D update: SWA_SCHEME_SPLIT or SWA_SCHEME_CTU
     int wetdry;            // split step with the shore solver (dry cells allowed)
     long long *gauge_row;  // device row counter of the fused gauge recording

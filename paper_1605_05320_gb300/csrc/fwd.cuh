@@ -21,7 +21,7 @@ struct FwdParams {
     int nblocks;
     int *err;          // device error word (ERR_* bits)
     int fwd_rows;      // FP32 strip height (rows per block), 0 = default
-    int keep_rest;     // FP32 2D: 1 computes wave-free rows in full (no skipping)
+    int keep_rest;     // FP32 2D: 1 computes units at rest in full
     const float *rest_tab;   // FP32 2D grid: rest CFL table of quiet units (null: none)
     unsigned char *umap;     // FP32 2D grid: marks of the strip step's units
     int umap_n;              // entries of umap

@@ -99,8 +99,8 @@ __global__ void __launch_bounds__(strip::kThreads, 4)
                 if (lane == 0) p.umap[u] = tag | UNIT_ACTIVE;
             }
         }
-        // Units with waves take the full path: quiet units cover the ocean
-        // at rest, and the strip loop without its row skipping is leaner.
+        // Units with waves take every row in full: a strip loop that tests
+        // rows for waves is slower, and quiet units cover the ocean at rest.
         if (CTU)
             strip::ctu_unit<ORD>(v, sx * strip::kOut, sy * rows, rows, s_nu[0], s_nu[1], p.g,
                                  ring[threadIdx.x >> 5], smax, bad);

@@ -7,8 +7,8 @@
 // Each loaded row (the output rows and two halo rows above and below) is
 // x-swept across the warp with shuffles, lane l solving and limiting edge
 // (l|l+1) once; the y-sweep of the x-swept rows runs in registers over a
-// sliding window of rows, each y-edge solved and limited once.  Rows are
-// loaded one iteration ahead of their use.  Ghost cells outside the grid are
+// sliding window of rows, each y-edge solved and limited once.  Rows reach
+// the warp through a ring in shared memory (cp.async).  Ghost cells outside the grid are
 // index-mapped on load (copy, or mirror with the normal momentum negated);
 // the x-sweep commutes with the y-mirror, so ghost rows may be x-swept like
 // any other.  Per edge the arithmetic is fwd_pair.cuh's, so results depend

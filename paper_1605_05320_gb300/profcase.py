@@ -8,7 +8,7 @@ and restores device memory between passes stays small:
   fwd   FP32 forward steps (fwd_f32_strips), ~120 MB on the device; the
         basin's initial state (the ocean at rest outside the source), or with
         `--active` seeded random momenta everywhere (no cell at rest)
-  ctu   FP32 unsplit forward steps with transverse waves (fwd_ctu_kernel),
+  ctu   FP32 unsplit forward steps with transverse waves (fwd_f32_strips, CTU),
         ~120 MB
   amr   two-level AMR steps on the basin: the 2048^2 coarse grid and 64
         patches refined by 4 around the source (coarse fluxes for the
