@@ -453,8 +453,12 @@ __global__ void __launch_bounds__(256) level_start_kernel(StartParams q) {
 
 // A patch's state from FP64 arrays, and to them (any output may be null): one
 // launch for all fields, the current buffer read from the level's clock.
+// Chained: many small patches are set or read one after the other, and a
+// launch's start is what each costs (480 patches set, stepped 180 times and
+// read: 16.2 / 14.6 ms).
 __global__ void patch_set_kernel(const double *eta, const double *hu, const double *hv, float *q0,
                                  float *q1, float *q2, size_t n) {
+    chain_begin();
     for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
          k += (size_t)gridDim.x * blockDim.x) {
         q0[k] = (float)eta[k];
@@ -469,6 +473,7 @@ struct PatchOut {
     double *h, *hu, *hv, *eta;
 };
 __global__ void patch_out_kernel(PatchOut p, size_t n) {
+    chain_begin();
     const int cur = p.clk->cur;
     for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
          k += (size_t)gridDim.x * blockDim.x) {
@@ -812,8 +817,8 @@ int swa_patches_set_state(swa_patchset *ps, int k, const double *eta, const doub
     const size_t nn = (size_t)ps->pd[k].nx * ps->pd[k].ny;
     float *const *q = ps->host_table[k].q[0];
     if (where == SWA_DEVICE) {
-        patch_set_kernel<<<ew_blocks(nn), 256, 0, st>>>(eta, hu, hv, q[0], q[1], q[2], nn);
-        TRY(cuda_check(cudaGetLastError(), "patch_set_kernel"));
+        TRY(cuda_check(launch_chained(patch_set_kernel, ew_blocks(nn), 256, 0, st, eta, hu, hv,
+                                      q[0], q[1], q[2], nn), "patch_set_kernel"));
     } else {   // one staging array: converted field by field
         const double *src[3] = {eta, hu, hv};
         for (int m = 0; m < 3; m++) {
@@ -856,15 +861,15 @@ int swa_patches_get_state(swa_patchset *ps, int k, double *h, double *hu, double
     p.hb = P.hb;
     if (where != SWA_HOST) {
         p.h = h; p.hu = hu; p.hv = hv; p.eta = eta;
-        patch_out_kernel<<<ew_blocks(nn), 256, 0, st>>>(p, nn);
-        return cuda_check(cudaGetLastError(), "patch_out_kernel");
+        return cuda_check(launch_chained(patch_out_kernel, ew_blocks(nn), 256, 0, st, p, nn),
+                          "patch_out_kernel");
     }
     double *dst[4] = {h, hu, hv, eta}, **field[4] = {&p.h, &p.hu, &p.hv, &p.eta};
     for (int m = 0; m < 4; m++) {   // one staging array: field by field
         if (!dst[m]) continue;
         for (int f = 0; f < 4; f++) *field[f] = f == m ? ps->staging : nullptr;
-        patch_out_kernel<<<ew_blocks(nn), 256, 0, st>>>(p, nn);
-        TRY(cuda_check(cudaGetLastError(), "patch_out_kernel"));
+        TRY(cuda_check(launch_chained(patch_out_kernel, ew_blocks(nn), 256, 0, st, p, nn),
+                       "patch_out_kernel"));
         TRY(cuda_check(cudaMemcpyAsync(dst[m], ps->staging, nn * 8, cudaMemcpyDeviceToHost, st),
                        "state download"));
         TRY(cuda_check(cudaStreamSynchronize(st), "state download"));
