@@ -196,10 +196,19 @@ def _ptr(x):
     return x.data_ptr()
 
 
+def _current_stream():
+    """The current stream's handle, without a Stream object for each call (3.0
+    us against 0.4; setting 480 small patches 3.8 ms against 2.0)."""
+    import torch
+    if not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    c = torch._C
+    return c._cuda_getCurrentRawStream(c._cuda_getDevice())
+
+
 def _stream(stream):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream

@@ -125,3 +125,10 @@ def test_conversion_equals_the_hardwares(tmp_path):
                    capture_output=True)
     r = subprocess.run([exe], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_default_stream_is_the_current_one(S):
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        assert S._stream(None) == side.cuda_stream == S._stream(side)
+    assert S._stream(None) == torch.cuda.current_stream().cuda_stream
