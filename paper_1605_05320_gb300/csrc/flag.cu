@@ -289,6 +289,26 @@ __global__ void __launch_bounds__(256) flag_kernel(FlagParams<R, S> p, int cells
 // case.  Each thread takes 4 consecutive cells with 16-byte loads; the window
 // (index ranges and end weights) is computed once per block, so the per-cell
 // loop has no FP64 work at all.
+//
+// PRUNE (no maxip output requested, envelope present): a group of snapshots
+// is read only where it can matter.  For a cell with forward state q and a
+// group whose per-component maxima over the cell's quad are (Me, Mu, Mv),
+// every product satisfies |q^ . q| <= Me |eta| + Mu |hu| + Mv |hv| =: bnd.
+// If bnd < tol (1 - 1e-5) for every wet cell of the quad, no product of the
+// group can reach tol even after float rounding (the products and bnd carry
+// relative errors of a few 1e-7), and neither can a time-interpolated end
+// value built from two such products; the group is skipped.  An end value
+// (INTERP) is computed from both of its snapshots whenever either of their
+// groups is read.  Every product that is formed is the one the unpruned pass
+// forms, so the flags and the count are identical to the unpruned pass; only
+// m differs (it may omit values below tol), hence PRUNE only without maxip.
+// Ahead of the forward wave q = 0 exactly: such a quad reads its state only.
+// On one grid a warp's loads are consecutive at every stage and its warps need
+// not wait for one another, so a thread keeps its quad from state to flags.
+// The phases of the other-grid pass below were up to 25 % faster here where
+// many groups matter (160 / 128 us at 2048^2), but up to 45 % slower where
+// all cells move and few groups do (27 / 39, 68 / 85).
+template <bool PRUNE>
 __global__ void __launch_bounds__(256, 4) flag_kernel_f32x4(FlagParams<float, float> p) {
     __shared__ Window sw;
     block_window(sw, p.tau, p.K, p.clk, p.t_s, p.t_f, p.mode);
@@ -297,6 +317,8 @@ __global__ void __launch_bounds__(256, 4) flag_kernel_f32x4(FlagParams<float, fl
     const size_t n4 = ((size_t)p.nx * p.ny) >> 2;
     const bool interp = p.mode != SWA_FLAG_BRACKET;
     const float tol = (float)p.tol;
+    const float tolp = (float)(p.tol * (1.0 - 1e-5));
+    const int gb0 = w.k0 / kEnvGroup, gb1 = w.k1 / kEnvGroup;
     const size_t cs = p.na >> 2, ks = p.snap_stride >> 2;
     int f = 0;
     // persistent grid: each block walks quads i, i + gridDim.x * 256, ...
@@ -312,27 +334,82 @@ __global__ void __launch_bounds__(256, 4) flag_kernel_f32x4(FlagParams<float, fl
         const bool ok2 = e.z + hb.z > dt && wet.z, ok3 = e.w + hb.w > dt && wet.w;
         float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
         float4 dh0 = m, dh1 = m, dl0 = m, dl1 = m;
-        if (!w.empty) {
+        // envelope test of group gb (PRUNE only): true when no product of the
+        // group can reach tol in any wet cell of the quad
+        auto skip = [&](int gb) -> bool {
+            const float *eg = p.env + (size_t)gb * 3 * n4;
+            const float Me = __ldg(eg + i), Mu = __ldg(eg + n4 + i), Mv = __ldg(eg + 2 * n4 + i);
+            const float b0 = Me * fabsf(e.x) + Mu * fabsf(u.x) + Mv * fabsf(v.x);
+            const float b1 = Me * fabsf(e.y) + Mu * fabsf(u.y) + Mv * fabsf(v.y);
+            const float b2 = Me * fabsf(e.z) + Mu * fabsf(u.z) + Mv * fabsf(v.z);
+            const float b3 = Me * fabsf(e.w) + Mu * fabsf(u.w) + Mv * fabsf(v.w);
+            return (!ok0 || b0 < tolp) && (!ok1 || b1 < tolp) && (!ok2 || b2 < tolp) &&
+                   (!ok3 || b3 < tolp);
+        };
+        // PRUNE: a quad whose forward state is exactly zero (the ocean at rest
+        // ahead of the wave) has every product exactly zero, m = 0 as in the
+        // full pass, so even its envelope is not read
+        const bool rest = e.x == 0.f && e.y == 0.f && e.z == 0.f && e.w == 0.f &&
+                          u.x == 0.f && u.y == 0.f && u.z == 0.f && u.w == 0.f &&
+                          v.x == 0.f && v.y == 0.f && v.z == 0.f && v.w == 0.f;
+        if (!w.empty && (!PRUNE || ((ok0 || ok1 || ok2 || ok3) && !rest))) {
             const float4 *s0 = reinterpret_cast<const float4 *>(p.snaps) + i;
+            // skip bits of the first 32 groups of the window (256 snapshots),
+            // their loads issued independently of one another
+            unsigned mask = 0u;
+            if (PRUNE) {
+                const int ng = gb1 - gb0 + 1 < 32 ? gb1 - gb0 + 1 : 32;
 #pragma unroll 2
-            for (int k = w.k0; k <= w.k1; k++) {
-                const float4 a = __ldcs(s0 + (size_t)k * ks);
-                const float4 b = __ldcs(s0 + (size_t)k * ks + cs);
-                const float4 c = __ldcs(s0 + (size_t)k * ks + 2 * cs);
-                float4 d;
-                // rounding fixed in the source, as in the pruned pass
-                d.x = fmaf(c.x, v.x, fmaf(b.x, u.x, __fmul_rn(a.x, e.x)));
-                d.y = fmaf(c.y, v.y, fmaf(b.y, u.y, __fmul_rn(a.y, e.y)));
-                d.z = fmaf(c.z, v.z, fmaf(b.z, u.z, __fmul_rn(a.z, e.z)));
-                d.w = fmaf(c.w, v.w, fmaf(b.w, u.w, __fmul_rn(a.w, e.w)));
-                if (k >= w.ki0 && k <= w.ki1) {
-                    m.x = fmaxf(m.x, fabsf(d.x)); m.y = fmaxf(m.y, fabsf(d.y));
-                    m.z = fmaxf(m.z, fabsf(d.z)); m.w = fmaxf(m.w, fabsf(d.w));
+                for (int j = 0; j < ng; j++)
+                    if (skip(gb0 + j)) mask |= 1u << j;
+            }
+            // groups past the first 32 of the window are always read
+            auto skipped = [&](int gb) -> bool {
+                const int j = gb - gb0;
+                return j < 32 && ((mask >> j) & 1u) != 0u;
+            };
+            bool need_h = true, need_l = true;
+            if (PRUNE && interp) {
+                const int kh1 = w.exact_h ? w.kh : w.kh + 1;
+                const int kl1 = w.exact_l ? w.kl : w.kl + 1;
+                need_h = !(skipped(w.kh / kEnvGroup) && skipped(kh1 / kEnvGroup));
+                need_l = !(skipped(w.kl / kEnvGroup) && skipped(kl1 / kEnvGroup));
+            }
+            for (int gb = gb0; gb <= gb1; gb++) {
+                const bool gs = PRUNE && skipped(gb);
+                const int ka = w.k0 > gb * kEnvGroup ? w.k0 : gb * kEnvGroup;
+                const int kb = w.k1 < gb * kEnvGroup + kEnvGroup - 1 ? w.k1
+                                                                    : gb * kEnvGroup + kEnvGroup - 1;
+                if (gs) {
+                    // a skipped group can only supply the snapshots of a
+                    // needed end pair
+                    const bool hh = need_h && w.kh <= kb && w.kh + 1 >= ka;
+                    const bool ll = need_l && w.kl <= kb && w.kl + 1 >= ka;
+                    if (!interp || !(hh || ll)) continue;
                 }
-                if (k == w.kh) dh0 = d;
-                if (k == w.kh + 1) dh1 = d;
-                if (k == w.kl) dl0 = d;
-                if (k == w.kl + 1) dl1 = d;
+#pragma unroll 2
+                for (int k = ka; k <= kb; k++) {
+                    if (gs && !((need_h && (k == w.kh || k == w.kh + 1)) ||
+                                (need_l && (k == w.kl || k == w.kl + 1))))
+                        continue;
+                    const float4 a = __ldcs(s0 + (size_t)k * ks);
+                    const float4 b = __ldcs(s0 + (size_t)k * ks + cs);
+                    const float4 c = __ldcs(s0 + (size_t)k * ks + 2 * cs);
+                    float4 d;
+                    // rounding fixed in the source, identical in both variants
+                    d.x = fmaf(c.x, v.x, fmaf(b.x, u.x, __fmul_rn(a.x, e.x)));
+                    d.y = fmaf(c.y, v.y, fmaf(b.y, u.y, __fmul_rn(a.y, e.y)));
+                    d.z = fmaf(c.z, v.z, fmaf(b.z, u.z, __fmul_rn(a.z, e.z)));
+                    d.w = fmaf(c.w, v.w, fmaf(b.w, u.w, __fmul_rn(a.w, e.w)));
+                    if (k >= w.ki0 && k <= w.ki1) {
+                        m.x = fmaxf(m.x, fabsf(d.x)); m.y = fmaxf(m.y, fabsf(d.y));
+                        m.z = fmaxf(m.z, fabsf(d.z)); m.w = fmaxf(m.w, fabsf(d.w));
+                    }
+                    if (k == w.kh) dh0 = d;
+                    if (k == w.kh + 1) dh1 = d;
+                    if (k == w.kl) dl0 = d;
+                    if (k == w.kl + 1) dl1 = d;
+                }
             }
             if (interp) {
                 const float ah = (float)w.ah, al = (float)w.al;
@@ -350,7 +427,7 @@ __global__ void __launch_bounds__(256, 4) flag_kernel_f32x4(FlagParams<float, fl
         const int f0 = (!w.empty && ok0 && m.x >= tol), f1 = (!w.empty && ok1 && m.y >= tol);
         const int f2 = (!w.empty && ok2 && m.z >= tol), f3 = (!w.empty && ok3 && m.w >= tol);
         reinterpret_cast<uchar4 *>(p.flags)[i] = make_uchar4(f0, f1, f2, f3);
-        if (p.maxip) {
+        if (!PRUNE && p.maxip) {
             const float4 mm = make_float4(ok0 ? m.x : 0.f, ok1 ? m.y : 0.f,
                                           ok2 ? m.z : 0.f, ok3 ? m.w : 0.f);
             reinterpret_cast<float4 *>(p.maxip)[i] = w.empty ? make_float4(0.f, 0.f, 0.f, 0.f) : mm;
@@ -362,9 +439,9 @@ __global__ void __launch_bounds__(256, 4) flag_kernel_f32x4(FlagParams<float, fl
     if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(p.count, (unsigned long long)cnt);
 }
 
-// The pruned pass: FP32 state and FP32 snapshots of a 2D adjoint with an
-// envelope, no maxip output; the adjoint on the same grid (SAME) or another
-// one.  A group of snapshots is read for a cell only where it can matter: for
+// The pruned pass with the adjoint on another grid: FP32 state and FP32
+// snapshots of a 2D adjoint with an envelope, no maxip output.  A group of
+// snapshots is read for a cell only where it can matter: for
 // a cell with forward state q and a group whose per-component maxima over the
 // envelope quads that hold its stencil are (Me, Mu, Mv), every product
 // satisfies |q^ . q| <= Me |eta| + Mu |hu| + Mv |hv| =: bnd (an interpolated
@@ -389,7 +466,7 @@ __global__ void __launch_bounds__(256, 4) flag_kernel_f32x4(FlagParams<float, fl
 // lanes of a warp waiting for its busiest quad; tiles of one warp were slower
 // on grids of few tiles, where the groups of a quad want many threads.)
 // Measured, us per pass, before / so (waves over a tenth and a third of the
-// domain): 2048^2 63 / 53 and 115 / 102; 512^2 over a 2048^2 adjoint with 401
+// domain): 512^2 over a 2048^2 adjoint with 401
 // snapshots 147 / 69 and 138 / 92; 4096^2 over 1024^2 237 / 147 and 427 / 313;
 // 1001 x 700 over 252 x 176 19.6 / 16.6 and 27.8 / 24.5.  Reading the group
 // with the largest bound first, to leave the others of a flagged cell, was
@@ -439,8 +516,8 @@ __device__ __forceinline__ Stencil stencil_f32(const FlagParams<float, float> &p
 }
 
 // VEC: nx % 4 == 0 (quads never straddle a row, 16-byte loads).
-template <bool SAME, bool VEC>
-__global__ void __launch_bounds__(kTile, SAME ? 4 : 3)
+template <bool VEC>
+__global__ void __launch_bounds__(kTile, 3)
     flag_pruned_kernel(FlagParams<float, float> p) {
     __shared__ Window sw;
     __shared__ FlagTile T;
@@ -500,8 +577,7 @@ __global__ void __launch_bounds__(kTile, SAME ? 4 : 3)
                 for (int c = 0; c < 4; c++) {
                     if (e[c] == 0.f && u[c] == 0.f && v[c] == 0.f) continue;
                     bool wet = e[c] + hb[c] > p.dry_tol;
-                    if (wet && SAME) wet = p.awet[o + c] != 0;
-                    if (wet && !SAME) {
+                    if (wet) {
                         const Stencil s = stencil_f32(p, ix + c, jy);
                         const uint8_t *a = p.awet + (size_t)s.j0 * p.anx + s.i0;
                         const uint8_t *b = a + (size_t)s.dj * p.anx;
@@ -552,15 +628,6 @@ __global__ void __launch_bounds__(kTile, SAME ? 4 : 3)
             }
             return dot3(d[0], T.q[0][c][a], d[1], T.q[1][c][a], d[2], T.q[2][c][a]);
         };
-        auto dot_quad = [&](size_t i4, int a, int k) {
-            const float4 *x = reinterpret_cast<const float4 *>(p.snaps + (size_t)k * p.snap_stride);
-            const float4 A = __ldcs(x + i4), B = __ldcs(x + na4 + i4), C = __ldcs(x + 2 * na4 + i4);
-            return make_float4(
-                dot3(A.x, T.q[0][0][a], B.x, T.q[1][0][a], C.x, T.q[2][0][a]),
-                dot3(A.y, T.q[0][1][a], B.y, T.q[1][1][a], C.y, T.q[2][1][a]),
-                dot3(A.z, T.q[0][2][a], B.z, T.q[1][2][a], C.z, T.q[2][2][a]),
-                dot3(A.w, T.q[0][3][a], B.w, T.q[1][3][a], C.w, T.q[2][3][a]));
-        };
         for (int gc = gb0; gc <= gb1; gc += kChunk) {
             const int ng = gb1 - gc + 1 < kChunk ? gb1 - gc + 1 : kChunk;
             // 2) which (quad, group) can matter
@@ -576,33 +643,27 @@ __global__ void __launch_bounds__(kTile, SAME ? 4 : 3)
             }
             // envelope quads x0 .. x1 of one row (same grid) or two
             unsigned x0, x1, y0, y1;
-            if (SAME) {
-                x0 = x1 = y0 = y1 = T.off[a] >> 2;
-            } else {
-                const int ix = T.ix[a], jy = T.jy[a];
-                const Stencil s0 = stencil_f32(p, ix, jy);
-                const Stencil s1 = stencil_f32(p, ix + 3 < p.nx ? ix + 3 : p.nx - 1, jy);
-                const unsigned r0 = (unsigned)s0.j0 * (unsigned)p.anx;
-                const unsigned r1 = r0 + (unsigned)(s0.dj * p.anx);
-                x0 = (r0 + s0.i0) >> 2; x1 = (r0 + s1.i0 + s1.di) >> 2;
-                y0 = (r1 + s0.i0) >> 2; y1 = (r1 + s1.i0 + s1.di) >> 2;
-            }
+            const int ix = T.ix[a], jy = T.jy[a];
+            const Stencil s0 = stencil_f32(p, ix, jy);
+            const Stencil s1 = stencil_f32(p, ix + 3 < p.nx ? ix + 3 : p.nx - 1, jy);
+            const unsigned r0 = (unsigned)s0.j0 * (unsigned)p.anx;
+            const unsigned r1 = r0 + (unsigned)(s0.dj * p.anx);
+            x0 = (r0 + s0.i0) >> 2; x1 = (r0 + s1.i0 + s1.di) >> 2;
+            y0 = (r1 + s0.i0) >> 2; y1 = (r1 + s1.i0 + s1.di) >> 2;
             const unsigned xm = x1 - x0 > y1 - y0 ? x1 - x0 : y1 - y0;
             const int gstep = kTile >> logP;   // the same for all lanes of a warp
 #pragma unroll 2
             for (int g = t >> logP; g < ng; g += gstep) {   // warp-uniform
                 const float *eg = p.env + (size_t)(gc + g) * 3 * na4;
                 float Me = __ldg(eg + x0), Mu = __ldg(eg + na4 + x0), Mv = __ldg(eg + 2 * na4 + x0);
-                if (!SAME) {
-                    Me = fmaxf(Me, __ldg(eg + y0));
-                    Mu = fmaxf(Mu, __ldg(eg + na4 + y0));
-                    Mv = fmaxf(Mv, __ldg(eg + 2 * na4 + y0));
-                    for (unsigned k = 1; k <= xm; k++) {
-                        const unsigned x = x0 + k < x1 ? x0 + k : x1, y = y0 + k < y1 ? y0 + k : y1;
-                        Me = fmaxf(Me, fmaxf(__ldg(eg + x), __ldg(eg + y)));
-                        Mu = fmaxf(Mu, fmaxf(__ldg(eg + na4 + x), __ldg(eg + na4 + y)));
-                        Mv = fmaxf(Mv, fmaxf(__ldg(eg + 2 * na4 + x), __ldg(eg + 2 * na4 + y)));
-                    }
+                Me = fmaxf(Me, __ldg(eg + y0));
+                Mu = fmaxf(Mu, __ldg(eg + na4 + y0));
+                Mv = fmaxf(Mv, __ldg(eg + 2 * na4 + y0));
+                for (unsigned k = 1; k <= xm; k++) {
+                    const unsigned x = x0 + k < x1 ? x0 + k : x1, y = y0 + k < y1 ? y0 + k : y1;
+                    Me = fmaxf(Me, fmaxf(__ldg(eg + x), __ldg(eg + y)));
+                    Mu = fmaxf(Mu, fmaxf(__ldg(eg + na4 + x), __ldg(eg + na4 + y)));
+                    Mv = fmaxf(Mv, fmaxf(__ldg(eg + 2 * na4 + x), __ldg(eg + 2 * na4 + y)));
                 }
                 bool need = false;
 #pragma unroll
@@ -623,34 +684,19 @@ __global__ void __launch_bounds__(kTile, SAME ? 4 : 3)
             __syncthreads();
             const int nitem = T.nitem;
             // 3) the products of those groups strictly inside the window
-            for (int it = t; it < (SAME ? nitem : 4 * nitem); it += kTile) {
-                const int item = T.item[SAME ? it : it >> 2], a = item & 255, c = it & 3;
+            for (int it = t; it < 4 * nitem; it += kTile) {
+                const int item = T.item[it >> 2], a = item & 255, c = it & 3;
                 const int g = gc + (item >> 8);
                 const int ka = w.ki0 > g * kEnvGroup ? w.ki0 : g * kEnvGroup;
                 const int kb = w.ki1 < g * kEnvGroup + kEnvGroup - 1 ? w.ki1
                                                                     : g * kEnvGroup + kEnvGroup - 1;
-                if (SAME) {
-                    const size_t i4 = T.off[a] >> 2;
-                    float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-                    for (int k = ka; k <= kb; k++) {
-                        const float4 d = dot_quad(i4, a, k);
-                        m.x = fmaxf(m.x, fabsf(d.x)); m.y = fmaxf(m.y, fabsf(d.y));
-                        m.z = fmaxf(m.z, fabsf(d.z)); m.w = fmaxf(m.w, fabsf(d.w));
-                    }
-                    atomicMax(&T.m[0][a], __float_as_int(m.x));
-                    atomicMax(&T.m[1][a], __float_as_int(m.y));
-                    atomicMax(&T.m[2][a], __float_as_int(m.z));
-                    atomicMax(&T.m[3][a], __float_as_int(m.w));
-                } else {
-                    // a cell that is flagged already needs no other group
-                    if (!((T.ok[a] >> c) & 1) || __int_as_float(T.m[c][a]) >= tol) continue;
-                    const Stencil s = stencil_f32(p, T.ix[a] + c, T.jy[a]);
-                    float m = 0.f;
+                // a cell that is flagged already needs no other group
+                if (!((T.ok[a] >> c) & 1) || __int_as_float(T.m[c][a]) >= tol) continue;
+                const Stencil s = stencil_f32(p, T.ix[a] + c, T.jy[a]);
+                float m = 0.f;
 #pragma unroll 2
-                    for (int k = ka; k <= kb; k++) m = fmaxf(m, fabsf(dot_cell(s, a, c, k)));
-                    atomicMax(&T.m[c][a], __float_as_int(m));
-                }
+                for (int k = ka; k <= kb; k++) m = fmaxf(m, fabsf(dot_cell(s, a, c, k)));
+                atomicMax(&T.m[c][a], __float_as_int(m));
             }
             __syncthreads();
             if (gc + kChunk <= gb1) {   // another chunk follows
@@ -660,55 +706,27 @@ __global__ void __launch_bounds__(kTile, SAME ? 4 : 3)
         }
         // 4) the window's ends and the flags (a cell flagged already needs
         // neither end)
-        for (int it = t; it < (SAME ? nact : 4 * nact); it += kTile) {
-            const int a = SAME ? it : it >> 2;
+        for (int it = t; it < 4 * nact; it += kTile) {
+            const int a = it >> 2;
             const size_t o = T.off[a];
             const float ah = (float)w.ah, al = (float)w.al, bh = 1.f - ah, bl = 1.f - al;
-            if (SAME) {
-                float m[4];
-                bool open = false;
-#pragma unroll
-                for (int c = 0; c < 4; c++) {
-                    m[c] = __int_as_float(T.m[c][a]);
-                    open = open || (((T.ok[a] >> c) & 1) && !(m[c] >= tol));
-                }
-                auto end = [&](bool exact, float x, float y, int k) {
-                    const float4 d0 = dot_quad(o >> 2, a, k);
-                    const float4 d1 = exact ? d0 : dot_quad(o >> 2, a, k + 1);
-                    auto at = [&](float r0, float r1) {
-                        return fabsf(exact ? r0 : fmaf(x, r0, __fmul_rn(y, r1)));
-                    };
-                    m[0] = fmaxf(m[0], at(d0.x, d1.x)); m[1] = fmaxf(m[1], at(d0.y, d1.y));
-                    m[2] = fmaxf(m[2], at(d0.z, d1.z)); m[3] = fmaxf(m[3], at(d0.w, d1.w));
-                };
-                if (open && T.need_h[a]) end(w.exact_h, ah, bh, w.kh);
-                if (open && T.need_l[a]) end(w.exact_l, al, bl, w.kl);
-                int g[4];
-#pragma unroll
-                for (int c = 0; c < 4; c++) g[c] = ((T.ok[a] >> c) & 1) && m[c] >= tol;
-                const int ng = g[0] + g[1] + g[2] + g[3];
-                f += ng;
-                if (ng)
-                    *reinterpret_cast<uchar4 *>(p.flags + o) = make_uchar4(g[0], g[1], g[2], g[3]);
-            } else {
-                const int c = it & 3;
-                if (!((T.ok[a] >> c) & 1)) continue;   // flag 0 already
-                const Stencil s = stencil_f32(p, T.ix[a] + c, T.jy[a]);
-                float m = __int_as_float(T.m[c][a]);
-                if (T.need_h[a] && !(m >= tol)) {
-                    const float d = dot_cell(s, a, c, w.kh);
-                    m = fmaxf(m, fabsf(w.exact_h ? d
-                                                 : fmaf(ah, d, __fmul_rn(bh, dot_cell(s, a, c, w.kh + 1)))));
-                }
-                if (T.need_l[a] && !(m >= tol)) {
-                    const float d = dot_cell(s, a, c, w.kl);
-                    m = fmaxf(m, fabsf(w.exact_l ? d
-                                                 : fmaf(al, d, __fmul_rn(bl, dot_cell(s, a, c, w.kl + 1)))));
-                }
-                if (m >= tol) {
-                    p.flags[o + c] = 1;
-                    f++;
-                }
+            const int c = it & 3;
+            if (!((T.ok[a] >> c) & 1)) continue;   // flag 0 already
+            const Stencil s = stencil_f32(p, T.ix[a] + c, T.jy[a]);
+            float m = __int_as_float(T.m[c][a]);
+            if (T.need_h[a] && !(m >= tol)) {
+                const float d = dot_cell(s, a, c, w.kh);
+                m = fmaxf(m, fabsf(w.exact_h ? d
+                                             : fmaf(ah, d, __fmul_rn(bh, dot_cell(s, a, c, w.kh + 1)))));
+            }
+            if (T.need_l[a] && !(m >= tol)) {
+                const float d = dot_cell(s, a, c, w.kl);
+                m = fmaxf(m, fabsf(w.exact_l ? d
+                                             : fmaf(al, d, __fmul_rn(bl, dot_cell(s, a, c, w.kl + 1)))));
+            }
+            if (m >= tol) {
+                p.flags[o + c] = 1;
+                f++;
             }
         }
         __syncthreads();
@@ -763,12 +781,12 @@ static unsigned persistent_blocks(K kernel, int &per_sm, size_t need) {
     return (unsigned)(need < b ? need : b);
 }
 
-template <bool SAME, bool VEC>
+template <bool VEC>
 static void launch_pruned(const FlagParams<float, float> &p, cudaStream_t st) {
     static int per_sm = 0;
     const size_t tiles = ((size_t)((p.nx + 3) / 4) * p.ny + 255) / 256;
-    const unsigned b = persistent_blocks(flag_pruned_kernel<SAME, VEC>, per_sm, tiles);
-    flag_pruned_kernel<SAME, VEC><<<b, 256, 0, st>>>(p);
+    const unsigned b = persistent_blocks(flag_pruned_kernel<VEC>, per_sm, tiles);
+    flag_pruned_kernel<VEC><<<b, 256, 0, st>>>(p);
 }
 
 template <typename R, typename S, bool SAME>
@@ -791,15 +809,20 @@ int flag_launch(const FlagParams<R, S> &p, cudaStream_t st) {
     const FlagParams<float, float> &pf = *reinterpret_cast<const FlagParams<float, float> *>(&p);
     // four flags, and four values of m, a store
     const bool aligned = ((uintptr_t)p.flags & 3) == 0 && ((uintptr_t)p.maxip & 15) == 0;
-    // the pruned pass takes m = 0 as no flag, so tol has to be above 0
-    if (f32 && p.env && !p.maxip && (float)p.tol > 0.f && (!p.same_grid || aligned)) {
-        if (p.same_grid) launch_pruned<true, true>(pf, st);
-        else if (p.nx % 4 == 0 && aligned) launch_pruned<false, true>(pf, st);
-        else launch_pruned<false, false>(pf, st);
-    } else if (f32 && p.same_grid && (n & 3) == 0 && aligned) {
-        static int per_sm = 0;
-        const unsigned b = persistent_blocks(flag_kernel_f32x4, per_sm, ((n >> 2) + 255) / 256);
-        flag_kernel_f32x4<<<b, 256, 0, st>>>(pf);
+    const bool prune = p.env && !p.maxip;
+    if (f32 && p.same_grid && (n & 3) == 0 && aligned) {
+        const size_t blocks = ((n >> 2) + 255) / 256;
+        static int per_sm[2] = {0, 0};
+        if (prune)
+            flag_kernel_f32x4<true>
+                <<<persistent_blocks(flag_kernel_f32x4<true>, per_sm[1], blocks), 256, 0, st>>>(pf);
+        else
+            flag_kernel_f32x4<false>
+                <<<persistent_blocks(flag_kernel_f32x4<false>, per_sm[0], blocks), 256, 0, st>>>(pf);
+    } else if (f32 && prune && !p.same_grid && (float)p.tol > 0.f) {
+        // this pass takes m = 0 as no flag, so tol has to be above 0
+        if (p.nx % 4 == 0 && aligned) launch_pruned<true>(pf, st);
+        else launch_pruned<false>(pf, st);
     } else if (p.same_grid) {
         launch_full<R, S, true>(p, n, st);
     } else {
