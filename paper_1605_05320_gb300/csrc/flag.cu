@@ -641,7 +641,7 @@ __global__ void __launch_bounds__(kTile, 3)
                 au[c] = in ? fabsf(T.q[1][c][a]) : 0.f;
                 av[c] = in ? fabsf(T.q[2][c][a]) : 0.f;
             }
-            // envelope quads x0 .. x1 of one row (same grid) or two
+            // envelope quads x0 .. x1 and y0 .. y1 of the stencil's two rows
             unsigned x0, x1, y0, y1;
             const int ix = T.ix[a], jy = T.jy[a];
             const Stencil s0 = stencil_f32(p, ix, jy);
