@@ -452,7 +452,8 @@ __global__ void __launch_bounds__(256) level_start_kernel(StartParams q) {
 }
 
 // A patch's state from FP64 arrays, and to them (any output may be null): one
-// launch for all fields, the current buffer read from the level's clock.
+// launch for all fields, the current buffer read from the level's clock (its
+// pointers selected, not indexed, as for a grid's state).
 // Chained: many small patches are set or read one after the other, and a
 // launch's start is what each costs (480 patches set, stepped 180 times and
 // read: 16.2 / 14.6 ms).
@@ -474,14 +475,21 @@ struct PatchOut {
 };
 __global__ void patch_out_kernel(PatchOut p, size_t n) {
     chain_begin();
-    const int cur = p.clk->cur;
+    const bool second = p.clk->cur != 0;
+    const float *q0 = second ? p.q[1][0] : p.q[0][0];
+    const float *q1 = second ? p.q[1][1] : p.q[0][1];
+    const float *q2 = second ? p.q[1][2] : p.q[0][2];
     for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
          k += (size_t)gridDim.x * blockDim.x) {
-        const double a = (double)p.q[cur][0][k];
-        if (p.h) p.h[k] = a + (double)p.hb[k];
-        if (p.eta) p.eta[k] = a;
-        if (p.hu) p.hu[k] = (double)p.q[cur][1][k];
-        if (p.hv) p.hv[k] = (double)p.q[cur][2][k];
+        if (p.h) {
+            const double a = (double)q0[k];
+            p.h[k] = a + (double)p.hb[k];
+            if (p.eta) p.eta[k] = a;
+        } else if (p.eta) {
+            p.eta[k] = (double)q0[k];
+        }
+        if (p.hu) p.hu[k] = (double)q1[k];
+        if (p.hv) p.hv[k] = (double)q2[k];
     }
 }
 
