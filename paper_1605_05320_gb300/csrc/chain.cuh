@@ -37,7 +37,9 @@ inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, s
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    if (e != cudaSuccess) cudaGetLastError();   // returned here, not left for a later check
+    return e;
 }
 
 }  // namespace swadj
