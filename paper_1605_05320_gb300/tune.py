@@ -1,26 +1,30 @@
 """Autotuner for the FP32 launch shapes of the step kernels: the strip height
 of a grid's step (16, 32 or 64 rows) and of a patch level's step (16 or 32
-rows).
+rows), or the height that the library chooses itself from the sizes (0).
 
 The launch shape changes only throughput, never results.  The tuner times
-each candidate with CUDA events on a few steps and keeps the faster one.  The
-choice is cached per device and shape signature (grid size, or the histogram
-of patch sizes of a level), in the process and in a JSON file that later
-processes read back (SWA_TUNE_CACHE names the file; the default lives in the
-user's cache directory; SWA_TUNE_CACHE="" keeps the cache in the process).
+each fixed height with CUDA events on a few steps, then the fastest of them
+in turn with the library's choice, and keeps that choice where it is no
+slower.  The result is cached per device, library and shape signature (grid
+size, or the histogram of patch sizes of a level), in the process and in a
+JSON file that later processes read back (SWA_TUNE_CACHE names the file; the
+default lives in the user's cache directory; SWA_TUNE_CACHE="" keeps the cache
+in the process).
 
 Tuning steps the object it is given: tune before setting the state you want
 to keep (or set it again afterwards; patch levels must be restarted).
 """
 from __future__ import annotations
 
+import functools
+import hashlib
 import json
 import os
 
 from . import swadj as S
 
-CANDIDATES = (32, 16)         # patch-level strip heights
-GRID_CANDIDATES = (32, 16, 64)  # grid strip heights
+CANDIDATES = (32, 16)         # fixed strip heights of a patch level
+GRID_CANDIDATES = (32, 16, 64)  # and of a grid
 _cache: dict = {}
 _loaded_from = None
 
@@ -75,6 +79,16 @@ def _device():
     return torch.cuda.get_device_name() if torch.cuda.is_available() else "cpu"
 
 
+@functools.lru_cache(maxsize=None)
+def _library() -> str:
+    """A digest of the library: heights timed on other kernels do not hold."""
+    try:
+        with open(S.LIB_PATH, "rb") as fh:
+            return hashlib.sha256(fh.read()).hexdigest()[:16]
+    except OSError:
+        return ""
+
+
 def _time(fn, steps):
     import torch
     fn(2)  # warm up (first launch sets kernel attributes)
@@ -88,9 +102,28 @@ def _time(fn, steps):
     return e0.elapsed_time(e1) / steps
 
 
+ROUNDS = 3          # timings of each height in turn
+RESOLVED_MS = 0.02  # CUDA events resolve about a microsecond: less decides nothing
+
+
+def _time_in_turn(apply, heights, run, steps):
+    """The least time per step of each height over some rounds in turn (a state
+    that changes as it is stepped is then the same for all), or None where
+    nothing can be measured: no device, or no work on it."""
+    import torch
+    if not torch.cuda.is_available():
+        return None
+    best = [float("inf")] * len(heights)
+    for _ in range(ROUNDS):
+        for k, rows in enumerate(heights):
+            apply(rows)
+            best[k] = min(best[k], _time(run, steps))
+    return best if min(best) * steps >= RESOLVED_MS else None
+
+
 def _choose(key, candidates, apply, run, steps):
     _load()
-    k = _key(key)
+    k = _key([_library()] + key)
     if k not in _cache:
         best, best_t = None, None
         for rows in candidates:
@@ -98,6 +131,9 @@ def _choose(key, candidates, apply, run, steps):
             t = _time(run, steps)
             if best_t is None or t < best_t:
                 best, best_t = rows, t
+        t = _time_in_turn(apply, (0, best), run, steps)
+        if t is not None and t[0] <= t[1]:
+            best = 0
         _cache[k] = best
         _store()
     apply(_cache[k])
@@ -105,7 +141,8 @@ def _choose(key, candidates, apply, run, steps):
 
 
 def tune_grid(grid: "S.Grid", steps: int = 10) -> int:
-    """Pick the strip height for a FP32 grid; returns it and applies it."""
+    """Pick the strip height for a FP32 grid (0: the library's choice); returns
+    it and applies it."""
     key = [_device(), "grid", grid.desc.nx, grid.desc.ny]
     return _choose(key, GRID_CANDIDATES, lambda rows: S.swa_grid_set_strip_rows(grid.h, rows),
                    lambda n: grid.step(n, 1e300), steps)
@@ -122,7 +159,8 @@ def _level_signature(ps: "S.PatchSet", level: int):
 
 def tune_patches(ps: "S.PatchSet", steps: int = 5) -> dict:
     """Pick the strip height of every level of a patch set (levels must have
-    been started); returns {level: rows} and applies it."""
+    been started); returns {level: rows} (0: the library's choice) and applies
+    it."""
     out = {}
     for level in ps.levels:
         key = [_device()] + _level_signature(ps, level)
