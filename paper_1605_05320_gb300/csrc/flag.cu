@@ -128,8 +128,15 @@ __device__ __forceinline__ double lerp2(double a, double x, double b, double y) 
 // does not depend on the order.
 // Measured, us per pass: 2000 cells in 1D with 701 FP64 snapshots 185 with one
 // thread a cell, 26 so.
+// The FP32 pass on one grid waits for memory, so a thread has several snapshots
+// in flight.  Measured, us per pass, one / so: 511 x 509 with about 40 snapshots in
+// the window 59 / 34, 1001 x 999 142 / 101, 1D 10^6 cells 55 / 39.  The blocks per
+// SM are those whose registers hold that: 5 for FP32 (48 registers) 52 at 511 x
+// 509, and for FP64, which its units bound, 4 (56 registers) left 628 blocks of
+// 401 x 399 in two rounds, 104 against 96.
 template <typename R, typename S, bool SAME>
-__global__ void __launch_bounds__(256) flag_kernel(FlagParams<R, S> p, int cells) {
+__global__ void __launch_bounds__(256, sizeof(R) + sizeof(S) == 8 ? 4 : SAME ? 5 : 3)
+    flag_kernel(FlagParams<R, S> p, int cells) {
     using A = typename std::conditional<sizeof(R) == 4 && sizeof(S) == 4, float,
                                         double>::type;
     __shared__ Window sw;
@@ -215,7 +222,7 @@ __global__ void __launch_bounds__(256) flag_kernel(FlagParams<R, S> p, int cells
         A mm = A(0), e0 = A(0), e1 = A(0), e2 = A(0), e3 = A(0);
         if (!w.empty && !dry) {
             A dh0 = A(0), dh1 = A(0), dl0 = A(0), dl1 = A(0);
-            for (int k = w.k0 + seg; k <= w.k1; k += segs) {
+            auto snapshot = [&](int k) {
                 const S *s = p.snaps + (size_t)k * p.snap_stride;
                 A v0, v1, v2 = A(0);
                 if (SAME) {
@@ -237,6 +244,19 @@ __global__ void __launch_bounds__(256) flag_kernel(FlagParams<R, S> p, int cells
                 if (k == w.kh + 1) dh1 = d;
                 if (k == w.kl) dl0 = d;
                 if (k == w.kl + 1) dl1 = d;
+            };
+            if constexpr (SAME && sizeof(A) == 4) {
+                if (p.ncomp == 3) {
+#pragma unroll 4
+                    for (int k = w.k0 + seg; k <= w.k1; k += segs) snapshot(k);
+                } else {   // 8 at a time, a short last batch repeating its first
+                    for (int k = w.k0 + seg; k <= w.k1; k += 8 * segs)
+#pragma unroll
+                        for (int j = 0; j < 8; j++)
+                            snapshot(k + j * segs <= w.k1 ? k + j * segs : k);
+                }
+            } else {
+                for (int k = w.k0 + seg; k <= w.k1; k += segs) snapshot(k);
             }
             if (segs > 1) {   // the threads of a cell meet in shared memory
                 s_m[threadIdx.x] = m;
@@ -792,10 +812,14 @@ static void launch_pruned(const FlagParams<float, float> &p, cudaStream_t st) {
 template <typename R, typename S, bool SAME>
 static void launch_full(const FlagParams<R, S> &p, size_t n, cudaStream_t st) {
     static int per_sm = 0;
-    // fewer cells a block while the grid has under about four blocks per SM and
-    // every thread keeps 8 snapshots or more
+    // fewer cells a block while the grid has under two blocks per SM (one on
+    // another grid, where every thread of a cell forms its stencil) and every
+    // thread keeps 8 snapshots or more.  Measured, us per pass, 256 / 128 cells:
+    // FP32 1D 50000 cells (1.3 blocks per SM), 600 snapshots 88 / 56, 100000
+    // (2.6) 18.6 / 19.2; FP64 on another grid 256^2 (1.7) 43 / 52.
+    const size_t sms = persistent_blocks(flag_kernel<R, S, SAME>, per_sm, SIZE_MAX) / per_sm;
     int cells = 256;
-    while (cells > 8 && n / cells < 600 && 16 * (256 / cells) <= p.K) cells /= 2;
+    while (cells > 8 && n / cells < (SAME ? 2 : 1) * sms && 16 * (256 / cells) <= p.K) cells /= 2;
     const unsigned b = persistent_blocks(flag_kernel<R, S, SAME>, per_sm, (n + cells - 1) / cells);
     flag_kernel<R, S, SAME><<<b, 256, 0, st>>>(p, cells);
 }
