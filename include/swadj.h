@@ -302,7 +302,8 @@ int swa_snapstore_info(const swa_snapstore *store, int *count, double *tau_host,
  * and FP32 snapshots of a 2D adjoint grid, the same grid or another one), a
  * snapshot group is read for a cell only if its envelope bound on
  * |q^ . q| reaches tol (1 - 1e-5) there (on another grid: the largest
- * envelope entry over the quads of the cell's bilinear stencil; on
+ * envelope entry over the quads of the cell's bilinear stencil, except that
+ * up to 2^20 cells times snapshots the full pass is the faster one and runs; on
  * the adjoint's own grid flags_dev must be aligned to 4 bytes for this, else
  * the full pass runs);
  * the flags and the count are identical to the full pass (every product the

@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(256, 4) flag_kernel_f32x4(FlagParams<float, fl
 // rest ahead of the wave) nothing but the state is read.
 //
 // What bounds it is the latency of dependent loads (state, envelope, then
-// snapshots), with work in few places.  A block therefore takes a tile of 256
+// snapshots), with work in few places.  A block therefore takes a tile of up to 256
 // quads in phases: it loads the states, packs the quads that move into a
 // list, tests (quad, group) pairs spread over its threads, packs those that
 // can matter into a second list, and spreads these over its threads again,
@@ -491,7 +491,12 @@ __global__ void __launch_bounds__(256, 4) flag_kernel_f32x4(FlagParams<float, fl
 // 1001 x 700 over 252 x 176 19.6 / 16.6 and 27.8 / 24.5.  Reading the group
 // with the largest bound first, to leave the others of a flagged cell, was
 // slower (its extra phases cost more than the reads: 122 and 418 us).
-constexpr int kTile = 256;      // quads per tile, threads per block
+// A grid of few tiles takes smaller ones, with the same threads: the fewest quads
+// (32 to 256) whose tiles are still one wave of blocks.  Measured, us per pass,
+// all cells moving, 256 / 128 / 64 / 32 quads: 128^2 over 192^2, 150 snapshots 51 / 32 /
+// 23 / 18 (253 tiles of 32 at 180^2: 47 / 31 / 22 / 19); 256^2 over 384^2 41 / 27 / 22 /
+// 23 (512 tiles of 32); 700^2 over 1048^2 62 / 62 / 77 / 90.
+constexpr int kTile = 256;      // quads per tile at most, threads per block
 constexpr int kChunk = 32;      // snapshot groups tested at a time
 struct FlagTile {
     float q[3][4][kTile];       // eta, hu, hv of the packed quads' cells
@@ -538,7 +543,7 @@ __device__ __forceinline__ Stencil stencil_f32(const FlagParams<float, float> &p
 // VEC: nx % 4 == 0 (quads never straddle a row, 16-byte loads).
 template <bool VEC>
 __global__ void __launch_bounds__(kTile, 3)
-    flag_pruned_kernel(FlagParams<float, float> p) {
+    flag_pruned_kernel(FlagParams<float, float> p, int tile) {
     __shared__ Window sw;
     __shared__ FlagTile T;
     const int t = threadIdx.x, lane = t & 31;
@@ -557,7 +562,7 @@ __global__ void __launch_bounds__(kTile, 3)
     const int gl0 = w.kl / kEnvGroup, gl1 = kl1 / kEnvGroup;
     const size_t na = p.na, na4 = na >> 2;
     int f = 0;
-    for (unsigned q0th = blockIdx.x * kTile; q0th < quads; q0th += gridDim.x * kTile) {
+    for (unsigned q0th = blockIdx.x * tile; q0th < quads; q0th += gridDim.x * tile) {
         if (t == 0) { T.nact = 0; T.nitem = 0; }
         __syncthreads();
         // 1) states; every flag starts at 0
@@ -566,7 +571,7 @@ __global__ void __launch_bounds__(kTile, 3)
         float e[4], u[4], v[4];
         int jy = 0, ix = 0;
         unsigned o = 0;
-        if (quad < quads) {
+        if (t < tile && quad < quads) {
             jy = (int)(quad / (unsigned)nq);
             ix = 4 * (int)(quad - (unsigned)jy * (unsigned)nq);
             o = (unsigned)jy * (unsigned)p.nx + (unsigned)ix;
@@ -804,9 +809,12 @@ static unsigned persistent_blocks(K kernel, int &per_sm, size_t need) {
 template <bool VEC>
 static void launch_pruned(const FlagParams<float, float> &p, cudaStream_t st) {
     static int per_sm = 0;
-    const size_t tiles = ((size_t)((p.nx + 3) / 4) * p.ny + 255) / 256;
-    const unsigned b = persistent_blocks(flag_pruned_kernel<VEC>, per_sm, tiles);
-    flag_pruned_kernel<VEC><<<b, 256, 0, st>>>(p);
+    const size_t quads = (size_t)((p.nx + 3) / 4) * p.ny;
+    const size_t wave = persistent_blocks(flag_pruned_kernel<VEC>, per_sm, SIZE_MAX);
+    int tile = 32;
+    while (tile < kTile && (quads + tile - 1) / tile > wave) tile *= 2;
+    const size_t tiles = (quads + tile - 1) / tile;
+    flag_pruned_kernel<VEC><<<(unsigned)(tiles < wave ? tiles : wave), kTile, 0, st>>>(p, tile);
 }
 
 template <typename R, typename S, bool SAME>
@@ -823,6 +831,14 @@ static void launch_full(const FlagParams<R, S> &p, size_t n, cudaStream_t st) {
     const unsigned b = persistent_blocks(flag_kernel<R, S, SAME>, per_sm, (n + cells - 1) / cells);
     flag_kernel<R, S, SAME><<<b, 256, 0, st>>>(p, cells);
 }
+
+// Cells times snapshots up to which a pass over another grid reads every
+// snapshot: the phases of the pruned pass, one waiting for the other, take longer
+// than the products then.  Measured, us per pass, full / pruned (waves over a
+// tenth and all of the domain): 64^2, 10 snapshots 12 / 12 and 12, 150 snapshots
+// 14 / 14 and 20; 300^2, 10 snapshots (0.9 M) 12 / 12 and 14; 180^2, 41 snapshots
+// (1.3 M) 14 / 13 and 14, 720^2 adjoint 20 / 13 and 15.
+constexpr size_t kFullProducts = 1 << 20;
 
 template <typename R, typename S>
 int flag_launch(const FlagParams<R, S> &p, cudaStream_t st) {
@@ -843,7 +859,7 @@ int flag_launch(const FlagParams<R, S> &p, cudaStream_t st) {
         else
             flag_kernel_f32x4<false>
                 <<<persistent_blocks(flag_kernel_f32x4<false>, per_sm[0], blocks), 256, 0, st>>>(pf);
-    } else if (f32 && prune && !p.same_grid && (float)p.tol > 0.f) {
+    } else if (f32 && prune && !p.same_grid && n * p.K > kFullProducts && (float)p.tol > 0.f) {
         // this pass takes m = 0 as no flag, so tol has to be above 0
         if (p.nx % 4 == 0 && aligned) launch_pruned<true>(pf, st);
         else launch_pruned<false>(pf, st);
