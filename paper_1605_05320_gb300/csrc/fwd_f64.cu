@@ -54,6 +54,12 @@ static int launch_sweep(const FwdParams<double> &p, int sms, cudaStream_t st) {
     return swadj_host::cuda_check(cudaGetLastError(), "fwd_f64_sweep");
 }
 
+// A 2D step runs as sweep passes, except on grids of a few long rows: there
+// the x-pass has fewer lines than a warp has lanes and its segments grow, while
+// the tiled kernel still takes one wave.
+// Measured, us per step with waves everywhere, tiles / sweeps: 1000 x 4 69 / 63
+// (segments of 2 cells), 2000 x 4 69 / 79 (4 cells), 4096 x 4 68 / 88 (7 cells;
+// wet/dry 137 / 161), 4096 x 8 (two waves of tiles) 107 / 89.
 template <bool WD>
 static int launch_sweeps(const FwdParams<double> &p, cudaStream_t st) {
     static int sms = 0;
@@ -63,6 +69,8 @@ static int launch_sweeps(const FwdParams<double> &p, cudaStream_t st) {
         cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
         sms = n > 0 ? n : 1;
     }
+    if (fwd_step_blocks<double>(p) <= sms && f64_segment(p.ny, p.nx, sms) > 3)
+        return launch_step<double, false, true, 32, 4, WD>(p, st);
     const int rc = launch_sweep<false, WD>(p, sms, st);
     return rc ? rc : launch_sweep<true, WD>(p, sms, st);
 }
