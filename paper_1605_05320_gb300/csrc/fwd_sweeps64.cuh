@@ -49,8 +49,9 @@ struct Edge {
 };
 
 // Velocities and sqrt(h) of a cell.  moving = false: its momenta are zero in
-// every lane of the warp, and sqrt(h) is left to an edge that needs it.
-template <bool WD>
+// every lane of the warp, and sqrt(h) is left to an edge that needs it.  A 1D
+// grid (TWO_D false) has no tangential momentum.
+template <bool WD, bool TWO_D = true>
 __device__ __forceinline__ Cell derive(double tol, double h, double mn, double mt, double eta,
                                        double b, bool moving) {
     Cell c;
@@ -60,12 +61,14 @@ __device__ __forceinline__ Cell derive(double tol, double h, double mn, double m
     if (moving && (!WD || h > tol)) {
         const Recip r = recip(h);
         c.un = div(mn, r);
-        c.ut = div(mt, r);
         c.sq = root(h);
         c.fn = mn * c.un;
-        c.ft = mn * c.ut;
         c.wn = c.sq * c.un;
-        c.wt = c.sq * c.ut;
+        if (TWO_D) {
+            c.ut = div(mt, r);
+            c.ft = mn * c.ut;
+            c.wt = c.sq * c.ut;
+        }
     }
     return c;
 }
@@ -412,7 +415,7 @@ __global__ void __launch_bounds__(32) fwd_f64_line(FwdParams<double> p) {
         const int o = ghost_index(i, p.nx, p.bc.lo_x, p.bc.hi_x, &flip);
         const double h = q0[o], b = p.bath[o];
         const double m = flip ? -q1[o] : q1[o];
-        const Cell c = derive<WD>(tol, h, m, 0.0, h + b, b, true);
+        const Cell c = derive<WD, false>(tol, h, m, 0.0, h + b, b, true);
         Cell r;
         r.h = dn(c.h); r.mn = dn(c.mn); r.mt = 0.0; r.eta = dn(c.eta); r.un = dn(c.un);
         r.ut = 0.0; r.sq = dn(c.sq); r.b = dn(c.b);
