@@ -8,8 +8,12 @@ namespace swadj {
 template <typename R, bool TWO_D, int TX, int TY>
 static int launch_adj(const AdjParams<R> &p, cudaStream_t st) {
     dim3 grid((p.nx + TX - 1) / TX, TWO_D ? (p.ny + TY - 1) / TY : 1);
+    // Measured, us per step in 1D, plain / chained: 8000 cells 16.1 / 13.4, 85000
+    // (665 blocks) 38 / 33, 90000 (704) 37 / 59, 150000 (1172) 55 / 58, 160000 59 / 59
+    static int wave = 0;
     return swadj_host::cuda_check(
-        launch_chained(adj_step_kernel<R, TWO_D, TX, TY>, grid, dim3(TX, TY), 0, st, p),
+        swadj_host::launch_spread(adj_step_kernel<R, TWO_D, TX, TY>, wave, 7, grid,
+                                  dim3(TX, TY), 0, st, p),
         "adj_step_kernel<double>");
 }
 

@@ -11,12 +11,12 @@
 // Measured, us per step, plain / chained: FP32 forward 64^2 12.3 / 10.3, 512^2
 // at rest outside the source 15.0 / 12.7, 2048^2 37.3 / 35.0 and with waves
 // everywhere 71.8 / 70.0; FP32 adjoint 512^2 8.2 / 5.8, 2048^2 early 19.9 / 17.5
-// and late 36.4 / 34.4.  Not chained are the kernels that the FP64 units bound, with
-// more than one block per SM: the blocks of a chained kernel take the slots that
-// become free first, so that some SMs hold more than their share and the FP64 units
-// of others idle (FP64 adjoint sweeps, 512^2 late: 103 plain, 140 chained; FP64
-// forward sweeps, whose units come from a counter once a block is placed, 256 x
-// 200: 101 and 117; FP64 unsplit step, 210 x 136: 108 and 145).  The FP64 1D step, in
+// and late 36.4 / 34.4.  The blocks of a chained kernel take the slots that become
+// free first, so that some SMs can hold more than their share while others idle.
+// The FP64 sweeps, which the FP64 units bound, are not chained for that (adjoint,
+// 512^2 late: 103 plain, 140 chained; forward, whose units come from a counter once a
+// block is placed, 256 x 200: 101 and 117), and kernels whose blocks take one share
+// of the work each are chained by their number (launch_spread).  The FP64 1D step, in
 // blocks of one warp, is chained at all sizes (2000 cells 12.9 and 11.3, 100000 34.2
 // and 32.2).
 #pragma once

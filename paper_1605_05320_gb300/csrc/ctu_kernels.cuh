@@ -333,24 +333,17 @@ int ctu_launch(FwdParams<R> p, cudaStream_t st, const char *name) {
     if (rc) return rc;
     dim3 grid((p.nx + TX - 1) / TX, (p.ny + TY - 1) / TY);
     p.nblocks = (int)(grid.x * grid.y);
-    // Chained with one block per SM at most: the blocks of a chained kernel take
-    // the slots that become free first, two or three on one SM while another has
-    // none, and the FP64 units bound this kernel.
-    // Measured, us per step, plain / chained: 128 x 100 (104 blocks) 72 / 70, 210 x
-    // 136 (238) 108 / 145, 250 x 136 (272) 109 / 146, 300 x 200 (475) 216 / 236, 400 x
-    // 200 (625) 298 / 290, 500 x 500 (2016) 735 / 733.
-    static int sms = 0;
-    if (sms == 0) {
-        int dev = 0, n = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        sms = n > 0 ? n : 1;
-    }
-    if (p.nblocks <= sms)
-        return swadj_host::cuda_check(
-            launch_chained(fwd_ctu_kernel<R, TX, TY>, grid, dim3(TX, TY), smem, st, p), name);
-    fwd_ctu_kernel<R, TX, TY><<<grid, dim3(TX, TY), smem, st>>>(p);
-    return swadj_host::cuda_check(cudaGetLastError(), name);
+    // Chained up to half the resident blocks only: the FP64 units bound this
+    // kernel, which feels blocks that crowd some SMs at more blocks too.
+    // Measured, us per step, plain / chained: 128 x 100 (104 blocks) 72 / 70, 130 x
+    // 136 (153) 108 / 104, 210 x 136 (238) 108 / 145, 250 x 136 (272) 109 / 146, 300 x
+    // 200 (475) 216 / 236, 400 x 200 (625) 298 / 290, 500 x 500 (2016) 735 / 733.
+    constexpr int kAnyBlocks = 1 << 20;
+    static int wave = 0;
+    return swadj_host::cuda_check(
+        swadj_host::launch_spread(fwd_ctu_kernel<R, TX, TY>, wave, kAnyBlocks, grid, dim3(TX, TY),
+                                  smem, st, p),
+        name);
 }
 
 template <int TX, int TY>

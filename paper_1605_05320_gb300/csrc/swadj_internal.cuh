@@ -180,4 +180,27 @@ namespace swadj_host {
 int set_error(int code, const char *fmt, ...);
 int cuda_check(cudaError_t e, const char *what);
 int *error_word();  // device address of the error word of the current device
+
+// Launches a kernel whose blocks take one share of the work each: chained where
+// the next launch's blocks all fit beside this one's, or nearly fill the GPU
+// themselves, and plainly where they are between half and `eighths` / 8 of the
+// resident blocks.  There the blocks of a chained kernel take the slots that
+// become free first, and some SMs hold more than their share while others have
+// none.  wave: the caller's static for the kernel's resident blocks.
+template <typename... P, typename... A>
+inline cudaError_t launch_spread(void (*kernel)(P...), int &wave, int eighths, dim3 grid,
+                                 dim3 block, size_t smem, cudaStream_t st, const A &...args) {
+    if (wave == 0) {
+        int dev = 0, sms = 0, per_sm = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block.x * block.y, smem);
+        wave = (sms > 0 ? sms : 1) * (per_sm > 0 ? per_sm : 1);
+    }
+    const long long b = (long long)grid.x * grid.y;
+    if (2 * b <= wave || 8 * b >= (long long)eighths * wave)
+        return swadj::launch_chained(kernel, grid, block, smem, st, args...);
+    kernel<<<grid, block, smem, st>>>(P(args)...);
+    return cudaGetLastError();
+}
 }  // namespace swadj_host
