@@ -85,6 +85,18 @@ def fits(used_bytes, n, budget_bytes, precision=S.SWA_FP32):
     return used_bytes + Server.footprint(n, precision) <= budget_bytes
 
 
+def strip_rows(sizes, warps):
+    """Strip height for small grids (n x n for n in sizes) that step side by
+    side: 0, the library's choice for a grid that steps alone (low strips, many
+    halo rows), until their strips of 16 rows are as many as the GPU's resident
+    warps; 16 from there, where the halo rows' work counts and not one step's
+    latency.  Results do not depend on it.
+    Measured, ms for 16 requests at once, 0 / 16 rows: 512^2 78 / 53, 512^2 and
+    1024^2 134 / 116; one request 9.1 / 10.3."""
+    units = sum(-(-n // 28) * -(-n // 16) for n in sizes)
+    return 16 if units >= warps else 0
+
+
 class ResidentAdjoint:
     """The adjoint for one target, solved once, snapshots kept on device."""
 
@@ -137,7 +149,14 @@ class Scenario:
         self.flags = torch.zeros(spec.n, dtype=torch.uint8, device=device)
         self.enqueued = 0
         self.events = []
+        self.rows = 0
         self.bytes = self.grid.nbytes + spec.n + self.series.numel() * 8
+
+    def set_rows(self, rows):
+        """Strip height of the macro steps enqueued from here on."""
+        if rows != self.rows:
+            S.swa_grid_set_strip_rows(self.grid.h, rows)
+            self.rows = rows
 
     def enqueue_macro(self, server):
         import torch
@@ -239,6 +258,8 @@ class Server:
         t0 = time.perf_counter()
         peak_active = 0
         peak_bytes = used
+        # resident warps of the step kernels: 4 blocks of 4 warps per SM
+        warps = 16 * torch.cuda.get_device_properties(self.device).multi_processor_count
         while pending or active:
             now = time.perf_counter() - t0
             # admit: the arrived request with the least work first (shortest
@@ -261,7 +282,9 @@ class Server:
             peak_bytes = max(peak_bytes, used)
             # keep every active scenario's queue topped up
             progressed = False
+            rows = strip_rows([sc.req.n for sc in active if sc.req.n <= SMALL], warps)
             for sc in active:
+                sc.set_rows(rows if sc.req.n <= SMALL else 0)
                 while sc.enqueued < sc.n_macro and sc.in_flight() < sc.ahead:
                     sc.enqueue_macro(self)
                     progressed = True
