@@ -120,14 +120,14 @@ __device__ __forceinline__ void ctu_unit(const View &v, int x0, int y0, int rows
         const float hb = R.v[sc][3][lane];
         sc = (sc + 1) & (kRing - 1);
         const Cell c = derive(eta, add(eta, hb), fx ? -mu : mu, fy ? -mv : mv);
-        const Edge w = xsolve<Nb1, true>(c, gh);
+        const Edge w = xsolve<true>(c, gh);
         const Edge Wn = j > y0 - 2 ? solve<true>(gh, turned(B), turned(c)) : W2;   // y-edge (j-1|j)
         float nb[3], np[3], nm[3], nx[3];   // row j: net, sums; row j-1: transverse x-correction
         Net N;
         auto row = [&](auto form) {
             constexpr bool SUB = decltype(form)::value;
             const Fluct f = fluct<SUB>(w);
-            const Net n = xnet<Nb1, SUB, ORD>(w, nux, f);
+            const Net n = xnet<SUB, ORD>(w, nux, f);
             nb[0] = mul(-nux, add(up(n.R0), n.L0));
             nb[1] = mul(-nux, add(up(n.R1), n.L1));
             nb[2] = mul(-nux, add(up(n.R2), n.L2));

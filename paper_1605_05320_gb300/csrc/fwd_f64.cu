@@ -10,12 +10,13 @@
 
 namespace swadj {
 
-template <typename R, bool PERT, bool TWO_D, int TX, int TY, bool WD = false>
-static int launch_step(FwdParams<R> p, cudaStream_t st) {
-    dim3 grid((p.nx + TX - 1) / TX, TWO_D ? (p.ny + TY - 1) / TY : 1);
+template <bool WD>
+static int launch_tiles(FwdParams<double> p, cudaStream_t st) {
+    dim3 grid((p.nx + 31) / 32, (p.ny + 3) / 4);
     p.nblocks = (int)(grid.x * grid.y);
     return swadj_host::cuda_check(
-        launch_chained(fwd_step_kernel<R, PERT, TWO_D, TX, TY, WD>, grid, dim3(TX, TY), 0, st, p),
+        launch_chained(fwd_step_kernel<double, false, true, 32, 4, WD>, grid, dim3(32, 4), 0, st,
+                       p),
         "fwd_step_kernel<double>");
 }
 
@@ -70,7 +71,7 @@ static int launch_sweeps(const FwdParams<double> &p, cudaStream_t st) {
         sms = n > 0 ? n : 1;
     }
     if (fwd_step_blocks<double>(p) <= sms && f64_segment(p.ny, p.nx, sms) > 3)
-        return launch_step<double, false, true, 32, 4, WD>(p, st);
+        return launch_tiles<WD>(p, st);
     const int rc = launch_sweep<false, WD>(p, sms, st);
     return rc ? rc : launch_sweep<true, WD>(p, sms, st);
 }
@@ -86,7 +87,7 @@ static int launch_line(const FwdParams<double> &p, cudaStream_t st) {
 
 template <>
 int fwd_launch_step<double>(const FwdParams<double> &p, cudaStream_t st) {
-    if (p.two_d && p.keep_input) return launch_step<double, false, true, 32, 4>(p, st);
+    if (p.two_d && p.keep_input) return launch_tiles<false>(p, st);
     if (p.two_d) return launch_sweeps<false>(p, st);
     return launch_line<false>(p, st);
 }

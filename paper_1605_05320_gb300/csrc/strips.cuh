@@ -38,70 +38,60 @@ struct View {
 __device__ __forceinline__ float dn(float x) { return __shfl_down_sync(kFull, x, 1); }
 __device__ __forceinline__ float up(float x) { return __shfl_up_sync(kFull, x, 1); }
 
-// How a lane reaches the cells and edges beside its own along x: one
-// column per lane, the neighbours are the lanes beside it (a policy, so the
-// x-sweep below serves other lane layouts too).  ok(): whether
-// the warp may take the SUB form, given this lane's edge (the nets of edges
-// (1|2) .. (29|30) are used).
-struct Nb1 {
-    static __device__ __forceinline__ float l(float x) { return up(x); }
-    static __device__ __forceinline__ float r(float x) { return dn(x); }
-    static __device__ __forceinline__ bool ok(const fp::Edge &w, int lane) {
-        return lane < 1 || lane > kLanes - 3 || fp::subsonic(w.s1, w.s3);
-    }
-};
+// Whether the warp may take the SUB form of a row, given this lane's x-edge (the
+// nets of edges (1|2) .. (29|30) are used).
+__device__ __forceinline__ bool x_subsonic(const fp::Edge &w, int lane) {
+    return lane < 1 || lane > kLanes - 3 || fp::subsonic(w.s1, w.s3);
+}
 
-// Net fluxes of a lane's x-edge(s) w, fetching the neighbour edges the
+// Net fluxes of a lane's x-edge w, fetching the neighbour edges the
 // limiter needs from the lanes beside it: in the SUB form only the upwind
 // values (wave 1 from the right edge, wave 3 from the left, both shear
 // strengths), otherwise both neighbours in full.
-template <class NB, bool SUB, int ORD>
+template <bool SUB, int ORD>
 __device__ __forceinline__ fp::Net xnet(const fp::Edge &w, float nu, const fp::Fluct &f) {
     fp::Up u1 = {}, u3 = {};
     if (SUB) {
         float b2l = w.b2, b2r = w.b2;
         if (ORD >= 2) {
-            u1.s = NB::r(w.s1); u1.vh = NB::r(w.vh); u1.b = NB::r(w.b1);
-            u3.s = NB::l(w.s3); u3.vh = NB::l(w.vh); u3.b = NB::l(w.b3);
-            b2l = NB::l(w.b2); b2r = NB::r(w.b2);
+            u1.s = dn(w.s1); u1.vh = dn(w.vh); u1.b = dn(w.b1);
+            u3.s = up(w.s3); u3.vh = up(w.vh); u3.b = up(w.b3);
+            b2l = up(w.b2); b2r = dn(w.b2);
         }
         return fp::net<true>(w, u1, u3, b2l, b2r, nu, ORD, f);
     }
     fp::Edge wl = w, wr = w;
     if (ORD >= 2) {
-        wl.s1 = NB::l(w.s1); wl.s3 = NB::l(w.s3); wl.vh = NB::l(w.vh);
-        wl.b1 = NB::l(w.b1); wl.b2 = NB::l(w.b2); wl.b3 = NB::l(w.b3);
-        wr.s1 = NB::r(w.s1); wr.s3 = NB::r(w.s3); wr.vh = NB::r(w.vh);
-        wr.b1 = NB::r(w.b1); wr.b2 = NB::r(w.b2); wr.b3 = NB::r(w.b3);
+        wl.s1 = up(w.s1); wl.s3 = up(w.s3); wl.vh = up(w.vh);
+        wl.b1 = up(w.b1); wl.b2 = up(w.b2); wl.b3 = up(w.b3);
+        wr.s1 = dn(w.s1); wr.s3 = dn(w.s3); wr.vh = dn(w.vh);
+        wr.b1 = dn(w.b1); wr.b2 = dn(w.b2); wr.b3 = dn(w.b3);
     }
     fp::upwind(w, wl, wr, u1, u3);
     return fp::net<false>(w, u1, u3, wl.b2, wr.b2, nu, ORD, f);
 }
 
-// The x-edge(s) a lane solves, between its cell and its right neighbour
+// The x-edge a lane solves, between its cell and its right neighbour
 // (x frame: mn = hu, mt = hv).
-template <class NB, bool RCP = false>
-__device__ __forceinline__ fp::Edge xsolve(const fp::Cell &c,
-                                                           float g_half) {
+template <bool RCP = false>
+__device__ __forceinline__ fp::Edge xsolve(const fp::Cell &c, float g_half) {
     fp::Cell r;
-    r.h = NB::r(c.h); r.mn = NB::r(c.mn); r.mt = c.mt; r.sq = NB::r(c.sq);
-    r.su = NB::r(c.su); r.sv = NB::r(c.sv); r.P = NB::r(c.P); r.T = NB::r(c.T);
-    r.eta = NB::r(c.eta);
+    r.h = dn(c.h); r.mn = dn(c.mn); r.mt = c.mt; r.sq = dn(c.sq);
+    r.su = dn(c.su); r.sv = dn(c.sv); r.P = dn(c.P); r.T = dn(c.T);
+    r.eta = dn(c.eta);
     return fp::solve<RCP>(g_half, c, r);
 }
 
-// The x-swept cell(s) in the y frame (mn = hv) from a lane's cell c and its
+// The x-swept cell in the y frame (mn = hv) from a lane's cell c and its
 // edge w: a cell takes R of the edge on its left and L of the edge on its
 // right.
-template <class NB, bool SUB, int ORD>
-__device__ __forceinline__ fp::Cell xsweep(const fp::Cell &c,
-                                                           const fp::Edge &w,
-                                                           float nux) {
-    const fp::Net n = xnet<NB, SUB, ORD>(w, nux, fp::fluct<SUB>(w));
+template <bool SUB, int ORD>
+__device__ __forceinline__ fp::Cell xsweep(const fp::Cell &c, const fp::Edge &w, float nux) {
+    const fp::Net n = xnet<SUB, ORD>(w, nux, fp::fluct<SUB>(w));
     const float mnu = -nux;
-    const float d0 = fp::mul(mnu, fp::add(NB::l(n.R0), n.L0));
-    const float d1 = fp::mul(mnu, fp::add(NB::l(n.R1), n.L1));
-    const float d2 = fp::mul(mnu, fp::add(NB::l(n.R2), n.L2));
+    const float d0 = fp::mul(mnu, fp::add(up(n.R0), n.L0));
+    const float d1 = fp::mul(mnu, fp::add(up(n.R1), n.L1));
+    const float d2 = fp::mul(mnu, fp::add(up(n.R2), n.L2));
     return fp::derive(fp::add(c.eta, d0), fp::add(c.h, d0), fp::add(c.mt, d2),
                       fp::add(c.mn, d1));
 }
@@ -209,9 +199,9 @@ __device__ __forceinline__ void strip_unit(const View &v, int x0, int y0, int ro
 #pragma unroll 1
     for (int k = 0; k < 4; k++) {   // rows y0 - 2 .. y0 + 1
         const Cell c = load();
-        const Edge w = xsolve<Nb1>(c, gh);
-        const Cell D = __all_sync(kFull, Nb1::ok(w, lane)) ? xsweep<Nb1, true, ORD>(c, w, nux)
-                                                           : xsweep<Nb1, false, ORD>(c, w, nux);
+        const Edge w = xsolve(c, gh);
+        const Cell D = __all_sync(kFull, x_subsonic(w, lane)) ? xsweep<true, ORD>(c, w, nux)
+                                                           : xsweep<false, ORD>(c, w, nux);
         if (k == 1) W1 = fp::solve(gh, C, D);
         if (k == 2) W2 = fp::solve(gh, C, D);
         A = B; B = C; C = D;
@@ -220,16 +210,16 @@ __device__ __forceinline__ void strip_unit(const View &v, int x0, int y0, int ro
 #pragma unroll UNR
     for (int j = y0 + 2; j <= jend; j++) {
         const Cell c = load();
-        const Edge w = xsolve<Nb1>(c, gh);
+        const Edge w = xsolve(c, gh);
         const Edge Wn = fp::solve(gh, B, C);   // y-edge (j-2|j-1)
         Cell D;
         fp::Net N;
-        if (__all_sync(kFull, Nb1::ok(w, lane) && (!out || fp::subsonic(W2.s1, W2.s3)))) {
-            D = xsweep<Nb1, true, ORD>(c, w, nux);
+        if (__all_sync(kFull, x_subsonic(w, lane) && (!out || fp::subsonic(W2.s1, W2.s3)))) {
+            D = xsweep<true, ORD>(c, w, nux);
             N = fp::net3(W1, W2, Wn, nuy, ORD, true);
             if (j > y0 + 2) finish(A, N1, N, j - 3);
         } else {
-            D = xsweep<Nb1, false, ORD>(c, w, nux);
+            D = xsweep<false, ORD>(c, w, nux);
             N = fp::net3(W1, W2, Wn, nuy, ORD, false);
             if (j > y0 + 2) finish(A, N1, N, j - 3);
         }
