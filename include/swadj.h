@@ -157,7 +157,9 @@ int swa_grid_set_strip_rows(swa_grid *grid, int rows);
  * (its CFL terms come from a table of the bathymetry's rest terms, formed
  * when the grid is created); on = 0 computes every unit in full.  Both give the same
  * state and time step (up to the sign of an exact zero); the switch exists
- * to show that and to time the step without the shortcut.  SWA_EINVAL for a
+ * to show that and to time the step without the shortcut.  In a hierarchy the
+ * averaging may bring waves to any unit of the coarse grid, so that units at rest
+ * are scanned and written again in each of its steps.  SWA_EINVAL for a
  * null grid or on not 0 or 1.
  */
 int swa_grid_set_rest_skip(swa_grid *g, int on);
@@ -209,9 +211,13 @@ int swa_grid_set_scheme(swa_grid *grid, int scheme);
 int swa_grid_set_wetdry(swa_grid *grid, int on);
 
 /*
- * Device pointers of the current state arrays (read-only use), for gauge or
- * diagnostic kernels of the caller.  Synchronises (the current buffer is
- * device-resident).  precision tells the element type (double or float).
+ * Device pointers of the current state arrays, for gauge or diagnostic kernels
+ * of the caller.  Read only: the FP32 2D step leaves units alone that it knows to
+ * be at rest, so that values written here would not be seen by it (swa_set_state
+ * is the way to change a state).  An FP64 2D step writes the new state into the
+ * arrays of the old one: a kernel that reads them on another stream has to be done
+ * before the next step.  Synchronises (the current buffer is device-resident).
+ * precision tells the element type (double or float).
  */
 int swa_grid_arrays(swa_grid *grid, const void **q0, const void **q1,
                     const void **q2, const void **bath, void *stream);

@@ -9,7 +9,7 @@
 // every lane has no waves and is not solved: far from the target the adjoint
 // is still exactly zero.
 // Measured, us per step early and late in the solve, tiles / sweeps: 512^2 212
-// and 223 / 58 and 88, 2048^2 3110 and 3120 / 260 and 353.
+// and 223 / 57 and 82, 2048^2 3110 and 3120 / 261 and 335.
 //
 // Every rounding operation is the FP64 reference's, in its order (an exact
 // zero is not added), so the state keeps the reference's bits.

@@ -232,8 +232,8 @@ static int grid_step_blocks(const swa_grid_desc *d) {
     return fwd_step_blocks<float>(p);
 }
 
-// Reduction slots for the smallest strip height the FP32 kernel accepts, or
-// for the unsplit step's tiles if there are more of those.
+// Reduction slots for the step kernel of most blocks: the FP32 strips at their
+// lowest height, the wet/dry and static steps' tiles, the FP64 unsplit step's.
 static int grid_max_blocks(const swa_grid_desc *d) {
     int b = grid_step_blocks(d);
     int w;

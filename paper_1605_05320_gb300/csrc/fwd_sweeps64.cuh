@@ -17,8 +17,8 @@
 // The x-pass reads buffer cur and writes the x-swept state to the other one,
 // the y-pass reads that and writes the new state back to buffer cur.
 // Measured, us per step, tiles / sweeps with quotients and roots of 3 and 6
-// FP64 operations / so (none): 512^2 (waves over 60 %) 721 / 216 / 160, 2048^2
-// 10400 / 2050 / 1462; 511 x 350 with wet/dry (a third land) 672 / 300 / 242.
+// FP64 operations / so (none): 512^2 (waves over 60 %) 721 / 216 / 154, 2048^2
+// 10400 / 2050 / 1448; 511 x 350 with wet/dry (a third land) 672 / 300 / 244.
 // The FP64 units stay what bounds it, with about 95 operations a cell and pass
 // (the cell's products formed once, not for both its edges: 3 % of it).
 //

@@ -1064,7 +1064,9 @@ __global__ void amr_avg_kernel(AvgParams p) {
         float *dst = (m.x < 0 ? *p.coarse : p.table[m.x]).q[pcur][k];
         dst[m.y] = block_sum<R>(S.q[fcur][k] + m.w, S.nx, r) * inv;
     }
-    // a unit at rest may have waves now; one that had waves stays marked
+    // a unit at rest may have waves now; one that had waves stays marked.  Every
+    // such mark goes, not only those under the level: the units at rest of a
+    // hierarchy's coarse grid are scanned once in each of its steps.
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < p.umap_n; k += gridDim.x * blockDim.x)
         if (p.umap[k] & UNIT_STILL) p.umap[k] = UNIT_UNKNOWN;
     if (blockIdx.x == 0 && threadIdx.x == 0) {

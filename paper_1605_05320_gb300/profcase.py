@@ -20,7 +20,7 @@ and restores device memory between passes stays small:
         envelope-pruned flag_kernel_f32x4) against a store of one snapshot
         every 100 adjoint steps, ~1.3 GB; `--full` requests m as well, which
         runs the full pass; `--adj-n 1024` puts the adjoint on a coarser
-        1024^2 grid (the pruned bilinear flag_kernel)
+        1024^2 grid (flag_pruned_kernel)
 
 Launch counts (for a profiler's -s / -c): `fwd` and `ctu` run 1 initial-CFL
 launch then `--steps` step launches; `amr` runs its set-up launches, then 11
