@@ -149,19 +149,23 @@ __global__ void state_out_kernel(StateOut<R> p, size_t n) {
     }
 }
 
-// Up to three arrays converted in one launch, dst[c] = (D) src[c].
+// Up to three arrays converted in one launch, dst[c] = (D) src[c], c the block's
+// row of the grid.  (A loop over the arrays in each thread ran the conversions of
+// absent ones too, which go through the FP64 units: an FP32 component of 2048^2 to
+// or from the host took 12 us longer.)
 template <typename S, typename D>
 struct Conv3 {
     const S *src[3];
     D *dst[3];
 };
 template <typename S, typename D>
-__global__ void conv3_kernel(Conv3<S, D> p, int nc, size_t n) {
+__global__ void conv3_kernel(Conv3<S, D> p, size_t n) {
+    const int c = blockIdx.y;
+    const S *src = c == 0 ? p.src[0] : c == 1 ? p.src[1] : p.src[2];
+    D *dst = c == 0 ? p.dst[0] : c == 1 ? p.dst[1] : p.dst[2];
     for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
          k += (size_t)gridDim.x * blockDim.x)
-#pragma unroll
-        for (int c = 0; c < 3; c++)
-            if (c < nc) p.dst[c][k] = (D)p.src[c][k];
+        dst[k] = (D)src[k];
 }
 
 __global__ void fill_zero_f64(double *p, size_t n) {
@@ -193,7 +197,7 @@ static int conv_in(const double *src, R *dst, const double *Bd, int mode, size_t
 
 template <typename S, typename D>
 static int conv3(const Conv3<S, D> &p, int nc, size_t n, cudaStream_t st) {
-    conv3_kernel<S, D><<<ew_blocks(n), 256, 0, st>>>(p, nc, n);
+    conv3_kernel<S, D><<<dim3(ew_blocks(n), nc), 256, 0, st>>>(p, n);
     return cuda_check(cudaGetLastError(), "conv3_kernel");
 }
 
