@@ -135,7 +135,7 @@ __device__ __forceinline__ double lerp2(double a, double x, double b, double y) 
 // 509, and for FP64, which its units bound, 4 (56 registers) left 628 blocks of
 // 401 x 399 in two rounds, 104 against 96.
 template <typename R, typename S, bool SAME>
-__global__ void __launch_bounds__(256, sizeof(R) + sizeof(S) == 8 ? 4 : SAME ? 5 : 3)
+__global__ void __launch_bounds__(256, !SAME ? 0 : sizeof(R) + sizeof(S) == 8 ? 4 : 5)
     flag_kernel(FlagParams<R, S> p, int cells) {
     using A = typename std::conditional<sizeof(R) == 4 && sizeof(S) == 4, float,
                                         double>::type;
@@ -820,16 +820,41 @@ static void launch_pruned(const FlagParams<float, float> &p, cudaStream_t st) {
 template <typename R, typename S, bool SAME>
 static void launch_full(const FlagParams<R, S> &p, size_t n, cudaStream_t st) {
     static int per_sm = 0;
-    // fewer cells a block while the grid has under two blocks per SM (one on
-    // another grid, where every thread of a cell forms its stencil) and every
-    // thread keeps 8 snapshots or more.  Measured, us per pass, 256 / 128 cells:
-    // FP32 1D 50000 cells (1.3 blocks per SM), 600 snapshots 88 / 56, 100000
-    // (2.6) 18.6 / 19.2; FP64 on another grid 256^2 (1.7) 43 / 52.
-    const size_t sms = persistent_blocks(flag_kernel<R, S, SAME>, per_sm, SIZE_MAX) / per_sm;
+    const size_t wave = persistent_blocks(flag_kernel<R, S, SAME>, per_sm, SIZE_MAX);
+    const size_t sms = wave / per_sm;
     int cells = 256;
-    while (cells > 8 && n / cells < (SAME ? 2 : 1) * sms && 16 * (256 / cells) <= p.K) cells /= 2;
-    const unsigned b = persistent_blocks(flag_kernel<R, S, SAME>, per_sm, (n + cells - 1) / cells);
-    flag_kernel<R, S, SAME><<<b, 256, 0, st>>>(p, cells);
+    if (SAME) {
+        // fewer cells a block while the grid has under two blocks per SM and every
+        // thread keeps 8 snapshots or more.  Measured, us per pass, 256 / 128 cells:
+        // FP32 1D 50000 cells (1.3 blocks per SM), 600 snapshots 88 / 56, 100000 (2.6)
+        // 18.6 / 19.2
+        while (cells > 8 && n / cells < 2 * sms && 16 * (256 / cells) <= p.K) cells /= 2;
+    } else {
+        // every thread of a cell forms its stencil, at the price of some snapshots:
+        // the cells of the least rounds times that and a thread's snapshots (and at
+        // about the same cost those that fill a round).  FP32 waits for memory, and a
+        // round is the resident blocks; FP64 is bound by its units, and a round is a
+        // block per SM.
+        // Measured, us per pass, 256 / 128 / 64 / 32 cells: FP32 200^2 over 300^2, 180
+        // snapshots 150 / 83 / 87 / 71, 300^2 over 75^2, 15 snapshots 14 / 16 / 17 / 24;
+        // FP64 230^2 over 57^2, 60 snapshots 138 / 112 / 124 / 148, 256^2 over 64^2, 15
+        // snapshots 44 / 52 / 60 / 88.
+        const bool f32 = sizeof(R) + sizeof(S) == 8;
+        const double setup = f32 ? 8.0 : 4.0;
+        const size_t round = f32 ? wave : sms;
+        double best = 0.0, margin = 1.0;
+        for (int c = 256; c >= 8 && (c == 256 || 4 * (256 / c) <= p.K); c /= 2) {
+            const size_t blocks = (n + c - 1) / c, rounds = (blocks + round - 1) / round;
+            const double cost = (double)rounds * (setup + (double)p.K * c / 256);
+            if (c == 256 || cost < margin * best) {
+                best = cost;
+                cells = c;
+                margin = blocks < round ? 1.05 : 0.97;
+            }
+        }
+    }
+    const size_t blocks = (n + cells - 1) / cells;
+    flag_kernel<R, S, SAME><<<(unsigned)(blocks < wave ? blocks : wave), 256, 0, st>>>(p, cells);
 }
 
 // Cells times snapshots up to which a pass over another grid reads every
