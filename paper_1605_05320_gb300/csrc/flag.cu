@@ -822,6 +822,7 @@ static void launch_full(const FlagParams<R, S> &p, size_t n, cudaStream_t st) {
     static int per_sm = 0;
     const size_t wave = persistent_blocks(flag_kernel<R, S, SAME>, per_sm, SIZE_MAX);
     const size_t sms = wave / per_sm;
+    const bool f32 = sizeof(R) + sizeof(S) == 8;
     int cells = 256;
     if (SAME) {
         // fewer cells a block while the grid has under two blocks per SM and every
@@ -829,27 +830,29 @@ static void launch_full(const FlagParams<R, S> &p, size_t n, cudaStream_t st) {
         // FP32 1D 50000 cells (1.3 blocks per SM), 600 snapshots 88 / 56, 100000 (2.6)
         // 18.6 / 19.2
         while (cells > 8 && n / cells < 2 * sms && 16 * (256 / cells) <= p.K) cells /= 2;
-    } else {
-        // every thread of a cell forms its stencil, at the price of some snapshots:
-        // the cells of the least rounds times that and a thread's snapshots (and at
-        // about the same cost those that fill a round).  FP32 waits for memory, and a
-        // round is the resident blocks; FP64 is bound by its units, and a round is a
-        // block per SM.
+    }
+    if (!SAME || !f32) {
+        // From there the cells of the least rounds times a thread's snapshots and the
+        // price of beginning a cell (on another grid every thread of it forms the
+        // stencil), and at about the same cost those that fill a round.  FP32 waits
+        // for memory, and a round is the resident blocks; FP64 is bound by its units,
+        // and a round is a block per SM.
         // Measured, us per pass, 256 / 128 / 64 / 32 cells: FP32 200^2 over 300^2, 180
         // snapshots 150 / 83 / 87 / 71, 300^2 over 75^2, 15 snapshots 14 / 16 / 17 / 24;
         // FP64 230^2 over 57^2, 60 snapshots 138 / 112 / 124 / 148, 256^2 over 64^2, 15
-        // snapshots 44 / 52 / 60 / 88.
-        const bool f32 = sizeof(R) + sizeof(S) == 8;
-        const double setup = f32 ? 8.0 : 4.0;
+        // snapshots 44 / 52 / 60 / 88; on one grid 351^2, 180 snapshots 193 / 172 / 173 /
+        // 171, 391^2 193 / 220 / 201 / 209.
+        const double setup = SAME ? 1.5 : f32 ? 8.0 : 4.0;
         const size_t round = f32 ? wave : sms;
+        const int most = cells;
         double best = 0.0, margin = 1.0;
-        for (int c = 256; c >= 8 && (c == 256 || 4 * (256 / c) <= p.K); c /= 2) {
+        for (int c = most; c >= 8 && (c == most || 4 * (256 / c) <= p.K); c /= 2) {
             const size_t blocks = (n + c - 1) / c, rounds = (blocks + round - 1) / round;
             const double cost = (double)rounds * (setup + (double)p.K * c / 256);
-            if (c == 256 || cost < margin * best) {
+            if (c == most || cost < margin * best) {
                 best = cost;
                 cells = c;
-                margin = blocks < round ? 1.05 : 0.97;
+                margin = !SAME && blocks < round ? 1.05 : 0.97;
             }
         }
     }
