@@ -132,8 +132,9 @@ __device__ __forceinline__ double lerp2(double a, double x, double b, double y) 
 // in flight.  Measured, us per pass, one / so: 511 x 509 with about 40 snapshots in
 // the window 59 / 34, 1001 x 999 142 / 101, 1D 10^6 cells 55 / 39.  The blocks per
 // SM are those whose registers hold that: 5 for FP32 (48 registers) 52 at 511 x
-// 509, and for FP64, which its units bound, 4 (56 registers) left 628 blocks of
-// 401 x 399 in two rounds, 104 against 96.
+// 509, and for FP64, which its units bound, 4 (56 registers) left 401 x 399 in blocks
+// of 256 cells in two rounds, 104 against 96.  On another grid the compiler's own 63
+// registers stand: a bound of 4 made it 64, and 332 x 1139 over 83 x 284 22.9 to 23.4.
 template <typename R, typename S, bool SAME>
 __global__ void __launch_bounds__(256, !SAME ? 0 : sizeof(R) + sizeof(S) == 8 ? 4 : 5)
     flag_kernel(FlagParams<R, S> p, int cells) {
